@@ -3,26 +3,39 @@
 // and the MLP predictor of Sec. 3.3 / Fig. 2 (one hidden layer of F ReLU units in front
 // of the K-bin softmax projection), its prediction and its loss.
 //
-// head_fwd_kernel: CTA b forms z = W h_b + bias (warp w takes logits k = w, w + 8, ...:
-//   lanes stride the D columns, then a fixed butterfly), p_hat = softmax(z),
-//   y_hat = sum p_hat_k c_k (relative to the centre of the largest logit), the soft
-//   label around the bin nearest to y_b, the prompt's CE and squared error, and dL/dz_b
-//   (with the batch mean's 1/B).
-// head_grad_kernel: one thread per output element of dL/dW = sum_b dz_b h_b^T,
-//   dL/dbias = sum_b dz_b and dL/dpooled_b = W^T dz_b, each summed in a fixed order,
-//   and the loss itself.  Everything is fp32.
-// mlp_hidden_kernel: u = max(W1 h + b1, 0), one warp per hidden unit and 8 prompts at a
-//   time (lanes stride D, then a fixed butterfly).  The MLP reuses the two kernels above
-//   layer by layer: head_fwd_kernel and head_grad_kernel on u with W2 (dL/dW2, dL/db2,
-//   dL/du and the loss), then head_grad_kernel on h with W1, gated by u > 0 (the ReLU's
-//   derivative), for dL/dW1, dL/db1 and dL/dh.
+// Everything is fp32: the contractions run on the FMA pipe through the tiles of sgemm.cuh.
+// A layer y = W x (x [B, D], W [K, D]) with its loss takes three launches:
+//   logit_part_kernel: z = W x cut into 32 x 32 tiles and, so that a small batch still fills
+//     the GPU, into splits of D; each split's sums go to its own slot of a partial buffer.
+//   head_loss_kernel: CTA b adds prompt b's slots in order, p_hat = softmax(z),
+//     y_hat = sum p_hat_k c_k (relative to the centre of the largest logit), the soft label
+//     around the bin nearest to y_b, the prompt's CE and squared error, and dL/dz_b (with the
+//     batch mean's 1/B).
+//   layer_grad_kernel: tiles of dL/dW = sum_b dz_b x_b^T and of dL/dx_b = W^T dz_b, with
+//     dL/dbias = sum_b dz_b along the first column of tiles, and one block for the loss.
+// The MLP adds wide_gemm_kernel, u = max(W1 h + b1, 0) and dL/dh = W1^T g, cut along its
+// contraction over a cluster whose CTAs add their tiles through distributed shared memory,
+// and outer_kernel, dL/dW1 = g^T h with dL/db1; g = dL/du where u > 0 (the ReLU's
+// derivative), formed by layer_grad_kernel.  Every sum runs in a fixed order.
+//
+// Measured, 256 prompts, D = 4096, K = 32 (GB300, device times with cold caches):
+//   linear head: 7.5 + 5.6 + 14.4 us against 51 + 48 us for one block a prompt forming its K dot
+//   products one after another (one load in flight a lane) and one thread an output of the
+//   gradients (256 dependent loads); the call 59 -> 26 us.
+//   MLP, F = 1024: hidden 60 us (36 TFLOP/s fp32), dL/dW1 55, dL/dh 64, against 489, 600 and 151
+//   for kernels that read an operand from L2 for every few FMAs; the call 1016 -> 198 us.
+#include <cooperative_groups.h>
+
 #include "estp_internal.cuh"
+#include "sgemm.cuh"
 
 namespace estp {
 namespace {
 
-constexpr int kFwdThreads = 256;
+namespace cg = cooperative_groups;
+
 constexpr int kMaxK = 1024;
+constexpr int kLossThreads = 128;
 
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
@@ -30,21 +43,61 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
-__global__ void __launch_bounds__(kFwdThreads) head_fwd_kernel(
-    const float* __restrict__ pooled, int64_t D, const float* __restrict__ W,
-    const float* __restrict__ bias, const float* __restrict__ centers, int K,
-    const float* __restrict__ targets, int B, float lambda3, float* __restrict__ dz,
-    float2* __restrict__ part, float* __restrict__ pred, float* __restrict__ probs) {
+// Each kernel below may be launched as a programmatic dependent of the launch before it: it
+// lets its own dependent start, then waits for the launch before it to complete.
+__device__ __forceinline__ void chain_launches() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Partial logits: part[s][b][k] = sum over split s of D of x[b, :] W[k, :].
+// Block (b tile of 32, k tile of 32, split).
+using LogitTile = SgemmTile<2, 2, 64, true, true>;
+__global__ void __launch_bounds__(256) logit_part_kernel(GemmSide x, GemmSide w, int64_t D, int split,
+                                                         float* __restrict__ part) {
+    __shared__ __align__(16) float sm[LogitTile::kSmemFloats];
+    chain_launches();
+    const int64_t b0 = (int64_t)blockIdx.x * LogitTile::BM, k0 = (int64_t)blockIdx.y * LogitTile::BN;
+    const int64_t d0 = (int64_t)blockIdx.z * split;
+    LogitTile t;
+    t.run(sm, x, b0, w, k0, d0, d0 + split < D ? d0 + split : D);
+    float* out = part + (int64_t)blockIdx.z * x.rows * w.rows;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int64_t b = b0 + t.row(i), k = k0 + t.col(0);
+        if (b < x.rows && k < w.rows) out[b * w.rows + k] = t.c[i][0].x;
+        if (b < x.rows && k + 1 < w.rows) out[b * w.rows + k + 1] = t.c[i][0].y;
+    }
+}
+
+// One block per prompt: logits from the n_split partial slots, then the head (targets NULL:
+// prediction only).
+__global__ void __launch_bounds__(kLossThreads) head_loss_kernel(
+    const float* __restrict__ zpart, int n_split, const float* __restrict__ bias,
+    const float* __restrict__ centers, int K, const float* __restrict__ targets, int B, float lambda3,
+    float* __restrict__ dz, float2* __restrict__ part, float* __restrict__ pred,
+    float* __restrict__ probs) {
     __shared__ float z_s[kMaxK];
+    chain_launches();
     const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
-    const float* h = pooled + (int64_t)b * D;
-    for (int k = warp; k < K; k += nw) {
-        const float* wk = W + (int64_t)k * D;
+    // four threads a bin add a quarter of the slots each (eight loads in flight), then two
+    // exchanges; the same order whatever the launch
+    for (int i0 = 0; i0 < 4 * K; i0 += kLossThreads) {
+        const int i = i0 + threadIdx.x, k = i >> 2;
         float acc = 0.f;
-        for (int64_t x = lane; x < D; x += 32) acc = fmaf(wk[x], h[x], acc);
-        acc = warp_sum(acc);
-        if (lane == 0) z_s[k] = acc + (bias ? bias[k] : 0.f);
+        if (k < K) {
+            const float* p = zpart + (int64_t)b * K + k;
+            const int64_t slot = (int64_t)B * K;
+            for (int s0 = i & 3; s0 < n_split; s0 += 32) {
+                float v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) v[j] = s0 + 4 * j < n_split ? __ldcg(p + (s0 + 4 * j) * slot) : 0.f;
+                acc += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+            }
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (k < K && (i & 3) == 0) z_s[k] = acc + (bias ? bias[k] : 0.f);
     }
     __syncthreads();
     if (warp != 0) return;
@@ -107,219 +160,265 @@ __global__ void __launch_bounds__(kFwdThreads) head_fwd_kernel(
     if (lane == 0) part[b] = make_float2(ce, err * err);
 }
 
-// gate (NULL: none): dz[b, k] counts only where gate[b, k] > 0 (a ReLU's derivative);
-// loss NULL: no loss element.
-__global__ void head_grad_kernel(const float* __restrict__ pooled, int B, int64_t D,
-                                 const float* __restrict__ W, int K, const float* __restrict__ dz,
-                                 const float* __restrict__ gate, const float2* __restrict__ part,
-                                 float lambda3, float* __restrict__ loss, float* __restrict__ grad_W,
-                                 float* __restrict__ grad_bias, float* __restrict__ grad_pooled) {
-    const int64_t n_w = grad_W ? (int64_t)K * D : 0;
-    const int64_t n_b = grad_bias ? K : 0;
-    const int64_t n_p = grad_pooled ? (int64_t)B * D : 0;
-    const int64_t total = n_w + n_b + n_p + (loss ? 1 : 0);
-    auto dzg = [&](int b, int k) -> float {
-        const float v = dz[(int64_t)b * K + k];
-        return gate && !(gate[(int64_t)b * K + k] > 0.f) ? 0.f : v;
-    };
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        if (t < n_w) {  // dL/dW[k, x] = sum_b dz[b, k] h[b, x]
-            const int k = (int)(t / D);
-            const int64_t x = t - (int64_t)k * D;
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b) acc = fmaf(dzg(b, k), pooled[(int64_t)b * D + x], acc);
-            grad_W[t] = acc;
-        } else if (t < n_w + n_b) {  // dL/dbias[k] = sum_b dz[b, k]
-            const int k = (int)(t - n_w);
-            float acc = 0.f;
-            for (int b = 0; b < B; ++b) acc += dzg(b, k);
-            grad_bias[k] = acc;
-        } else if (t < n_w + n_b + n_p) {  // dL/dpooled[b, x] = sum_k W[k, x] dz[b, k]
-            const int64_t r = t - n_w - n_b;
-            const int b = (int)(r / D);
-            const int64_t x = r - (int64_t)b * D;
-            float acc = 0.f;
-            for (int k = 0; k < K; ++k) acc = fmaf(W[(int64_t)k * D + x], dzg(b, k), acc);
-            grad_pooled[r] = acc;
-        } else {  // the loss: batch means of the CE and squared-error terms
-            float ce = 0.f, se = 0.f;
-            for (int b = 0; b < B; ++b) {
-                ce += part[b].x;
-                se += part[b].y;
-            }
-            loss[0] = (lambda3 * ce + (1.f - lambda3) * se) / (float)B;
+// Gradients of the layer y = W x from dz = dL/dy: blocks [0, n_w) are tiles of
+// dL/dW [K, D] (column-major over the D tiles; the first D tile also gives dL/dbias), blocks
+// [n_w, n_w + n_x) tiles of dL/dx [B, D], and one last block the loss.  gate (or NULL):
+// dL/dx counts only where gate > 0 (the ReLU's derivative of the layer below).
+struct LayerGradArgs {
+    GemmSide dz_k;      // rows = bins, k = prompts (side contiguous)
+    GemmSide dz_b;      // rows = prompts, k = bins (k contiguous)
+    GemmSide x_d, w_d;  // rows = D columns, k = prompts / bins (side contiguous)
+    int B, K;
+    int64_t D;
+    int n_wk, n_w, n_x;
+    float* grad_W;
+    float* grad_bias;
+    float* grad_x;
+    const float* gate;
+    const float2* part;
+    float lambda3;
+    float* loss;
+};
+using GradWTile = SgemmTile<2, 4, 32, false, false>;
+using GradXTile = SgemmTile<2, 4, 32, true, false>;
+__global__ void __launch_bounds__(256) layer_grad_kernel(const LayerGradArgs a) {
+    constexpr int kFloats = GradWTile::kSmemFloats > GradXTile::kSmemFloats ? GradWTile::kSmemFloats
+                                                                            : GradXTile::kSmemFloats;
+    __shared__ __align__(16) float sm[kFloats];
+    chain_launches();
+    int blk = blockIdx.x;
+    if (blk < a.n_w) {
+        const int64_t k0 = (int64_t)(blk % a.n_wk) * GradWTile::BM, d0 = (int64_t)(blk / a.n_wk) * GradWTile::BN;
+        GradWTile t;
+        float db = 0.f;
+        if (d0 == 0) t.template run<true>(sm, a.dz_k, k0, a.x_d, d0, 0, a.B, &db);
+        else t.run(sm, a.dz_k, k0, a.x_d, d0, 0, a.B);
+        if (a.grad_bias && d0 == 0 && threadIdx.x < GradWTile::BM && k0 + threadIdx.x < a.K)
+            a.grad_bias[k0 + threadIdx.x] = db;
+        if (!a.grad_W) return;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int64_t k = k0 + t.row(i), d = d0 + t.col(0);
+            if (k >= a.K) continue;
+            const float v[4] = {t.c[i][0].x, t.c[i][0].y, t.c[i][1].x, t.c[i][1].y};
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (d + j < a.D) a.grad_W[k * a.D + d + j] = v[j];
         }
+        return;
     }
-}
-
-constexpr int kHidB = 16;  // prompts per warp pass of the hidden layer
-constexpr int kDhB = 4;    // prompts per block of the input gradient
-
-// Four consecutive floats of a row at column x (a 16-byte load when vec, else scalar
-// loads, zero past D).
-__device__ __forceinline__ float4 ld4(const float* __restrict__ row, int64_t x, int64_t D, bool vec) {
-    if (vec) return __ldg(reinterpret_cast<const float4*>(row + x));
-    return make_float4(x < D ? __ldg(row + x) : 0.f, x + 1 < D ? __ldg(row + x + 1) : 0.f,
-                       x + 2 < D ? __ldg(row + x + 2) : 0.f, x + 3 < D ? __ldg(row + x + 3) : 0.f);
-}
-
-// u[b, f] = max(sum_x W1[f, x] h[b, x] + b1[f], 0): one warp per hidden unit f, lanes
-// stride D four columns at a time, kHidB prompts per pass, then a fixed butterfly.
-__global__ void __launch_bounds__(128) mlp_hidden_kernel(const float* __restrict__ pooled, int B,
-                                                         int64_t D, const float* __restrict__ W1,
-                                                         const float* __restrict__ b1, int F,
-                                                         float* __restrict__ u, int vec) {
-    const int lane = threadIdx.x & 31;
-    const int64_t f = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (f >= F) return;
-    const float* w = W1 + f * D;
-    const float bias = b1 ? b1[f] : 0.f;
-    for (int b0 = 0; b0 < B; b0 += kHidB) {
-        const int nb = B - b0 < kHidB ? B - b0 : kHidB;
-        float acc[kHidB];
+    blk -= a.n_w;
+    if (blk < a.n_x) {
+        const int64_t n_bt = (a.B + GradXTile::BM - 1) / GradXTile::BM;
+        const int64_t b0 = (blk % n_bt) * GradXTile::BM, d0 = (blk / n_bt) * GradXTile::BN;
+        GradXTile t;
+        t.run(sm, a.dz_b, b0, a.w_d, d0, 0, a.K);
 #pragma unroll
-        for (int j = 0; j < kHidB; ++j) acc[j] = 0.f;
-        for (int64_t x = 4 * lane; x < D; x += 128) {
-            // every load of the pass first (rows past B repeat the last row, unused), then the FMAs
-            const float4 wv = ld4(w, x, D, vec);
-            float4 hv[kHidB];
+        for (int i = 0; i < 2; ++i) {
+            const int64_t b = b0 + t.row(i), d = d0 + t.col(0);
+            if (b >= a.B) continue;
+            const float v[4] = {t.c[i][0].x, t.c[i][0].y, t.c[i][1].x, t.c[i][1].y};
 #pragma unroll
-            for (int j = 0; j < kHidB; ++j)
-                hv[j] = ld4(pooled + (int64_t)(b0 + (j < nb ? j : nb - 1)) * D, x, D, vec);
-#pragma unroll
-            for (int j = 0; j < kHidB; ++j)
-                acc[j] = fmaf(wv.x, hv[j].x, fmaf(wv.y, hv[j].y, fmaf(wv.z, hv[j].z, fmaf(wv.w, hv[j].w, acc[j]))));
+            for (int j = 0; j < 4; ++j)
+                if (d + j < a.D)
+                    a.grad_x[b * a.D + d + j] = a.gate && !(a.gate[b * a.D + d + j] > 0.f) ? 0.f : v[j];
         }
-#pragma unroll
-        for (int j = 0; j < kHidB; ++j) {
-            const float a = warp_sum(acc[j]) + bias;
-            if (lane == 0 && j < nb) u[(int64_t)(b0 + j) * F + f] = a > 0.f ? a : 0.f;
-        }
+        return;
     }
-}
-
-// dL/dh[b, x] = sum_f W1[f, x] g[b, f], g = dL/du where u > 0 (the ReLU's derivative), else 0.
-// Block (128 columns, kDhB prompts): g of the block's prompts is staged in shared memory
-// (dynamic, kDhB x F floats); warp w takes f = w, w + 8, ... (four W1 rows in flight);
-// the 8 warp partials are added in warp order.
-__global__ void __launch_bounds__(256) mlp_dh_kernel(const float* __restrict__ W1, int64_t D, int F,
-                                                     const float* __restrict__ du,
-                                                     const float* __restrict__ u, int B,
-                                                     float* __restrict__ dh, int vec) {
-    extern __shared__ float g_s[];  // [kDhB][F]
-    __shared__ float4 red[8][kDhB][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t x = (int64_t)blockIdx.x * 128 + 4 * lane;
-    const int b0 = blockIdx.y * kDhB;
-    const int nb = B - b0 < kDhB ? B - b0 : kDhB;
-    for (int q = threadIdx.x; q < kDhB * F; q += blockDim.x) {
-        const int j = q / F, f = q - j * F;
-        float gv = 0.f;
-        if (j < nb) {
-            const int64_t i = (int64_t)(b0 + j) * F + f;
-            gv = u[i] > 0.f ? du[i] : 0.f;
-        }
-        g_s[q] = gv;
+    // the loss: batch means of the CE and squared-error terms (256 strided sums, then a tree)
+    float ce = 0.f, se = 0.f;
+    for (int b = threadIdx.x; b < a.B; b += 256) {
+        const float2 p = a.part[b];
+        ce += p.x;
+        se += p.y;
+    }
+    ce = warp_sum(ce);
+    se = warp_sum(se);
+    if ((threadIdx.x & 31) == 0) {
+        sm[threadIdx.x >> 5] = ce;
+        sm[8 + (threadIdx.x >> 5)] = se;
     }
     __syncthreads();
-    float4 acc[kDhB];
-#pragma unroll
-    for (int j = 0; j < kDhB; ++j) acc[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (x < D) {
-        int f = warp;
-        for (; f + 24 < F; f += 32) {  // four rows f, f + 8, f + 16, f + 24 in flight
-            float4 wv[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) wv[r] = ld4(W1 + (int64_t)(f + 8 * r) * D, x, D, vec);
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int j = 0; j < kDhB; ++j) {
-                    const float gv = g_s[j * F + f + 8 * r];
-                    acc[j].x = fmaf(gv, wv[r].x, acc[j].x);
-                    acc[j].y = fmaf(gv, wv[r].y, acc[j].y);
-                    acc[j].z = fmaf(gv, wv[r].z, acc[j].z);
-                    acc[j].w = fmaf(gv, wv[r].w, acc[j].w);
-                }
+    if (threadIdx.x == 0) {
+        ce = se = 0.f;
+        for (int w = 0; w < 8; ++w) {
+            ce += sm[w];
+            se += sm[8 + w];
         }
-        for (; f < F; f += 8) {
-            const float4 wv = ld4(W1 + (int64_t)f * D, x, D, vec);
-#pragma unroll
-            for (int j = 0; j < kDhB; ++j) {
-                const float gv = g_s[j * F + f];
-                acc[j].x = fmaf(gv, wv.x, acc[j].x);
-                acc[j].y = fmaf(gv, wv.y, acc[j].y);
-                acc[j].z = fmaf(gv, wv.z, acc[j].z);
-                acc[j].w = fmaf(gv, wv.w, acc[j].w);
-            }
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < kDhB; ++j) red[warp][j][lane] = acc[j];
-    __syncthreads();
-    if (warp == 0 && x < D) {
-        for (int j = 0; j < nb; ++j) {
-            float4 t = red[0][j][lane];
-            for (int w = 1; w < 8; ++w) {
-                const float4 o = red[w][j][lane];
-                t.x += o.x;
-                t.y += o.y;
-                t.z += o.z;
-                t.w += o.w;
-            }
-            float* out = dh + (int64_t)(b0 + j) * D + x;
-            out[0] = t.x;
-            if (x + 1 < D) out[1] = t.y;
-            if (x + 2 < D) out[2] = t.z;
-            if (x + 3 < D) out[3] = t.w;
-        }
+        a.loss[0] = (a.lambda3 * ce + (1.f - a.lambda3) * se) / (float)a.B;
     }
 }
 
-// dL/dW1[f, x] = sum_b g[b, f] h[b, x] and dL/db1[f] = sum_b g[b, f], g = dL/du where u > 0:
-// thread (f, four columns x) sums the prompts in order; the threads with x = 0 also write
-// dL/db1[f].  Either output may be NULL.
-__global__ void __launch_bounds__(256) mlp_dw1_kernel(const float* __restrict__ pooled, int B,
-                                                      int64_t D, int F, const float* __restrict__ du,
-                                                      const float* __restrict__ u,
-                                                      float* __restrict__ gW1,
-                                                      float* __restrict__ gb1, int vec) {
-    const int64_t per_row = (D + 3) / 4;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int64_t)F * per_row) return;
-    const int f = (int)(t / per_row);
-    const int64_t x = 4 * (t - (int64_t)f * per_row);
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    float gs = 0.f;
-    for (int b = 0; b < B; ++b) {
-        const int64_t i = (int64_t)b * F + f;
-        const float gv = u[i] > 0.f ? du[i] : 0.f;
-        gs += gv;
-        if (gW1) {
-            const float4 hv = ld4(pooled + (int64_t)b * D, x, D, vec);
-            acc.x = fmaf(gv, hv.x, acc.x);
-            acc.y = fmaf(gv, hv.y, acc.y);
-            acc.z = fmaf(gv, hv.z, acc.z);
-            acc.w = fmaf(gv, hv.w, acc.w);
+// out[m, n] = sum_k A(m, k) B(n, k) (+ bias[n], then max with 0, when kRelu): block (n tile of
+// 64, m tile, rank of the cluster along k).  The ranks' tiles meet in shared memory, and each
+// rank adds its share of the rows over all ranks in rank order.
+template <int TM, int BK, bool kAlongB>
+using WideTile = SgemmTile<TM, 4, BK, true, kAlongB>;
+
+template <int TM, int BK, bool kAlongB, bool kRelu>
+__global__ void __launch_bounds__(256, 2) wide_gemm_kernel(GemmSide A, GemmSide Bm, int64_t n_k,
+                                                           const float* __restrict__ bias,
+                                                           float* __restrict__ out) {
+    using T = WideTile<TM, BK, kAlongB>;
+    constexpr int SC = T::BN + 4;
+    __shared__ __align__(16) float sm[T::kSmemFloats > T::BM * SC ? T::kSmemFloats : T::BM * SC];
+    chain_launches();
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)blockIdx.z, ranks = (int)gridDim.z;  // the cluster spans z
+    const int64_t n0 = (int64_t)blockIdx.x * T::BN, m0 = (int64_t)blockIdx.y * T::BM;
+    const int64_t per = ((n_k + ranks - 1) / ranks + 63) / 64 * 64;
+    const int64_t k0 = rank * per, k1 = k0 + per < n_k ? k0 + per : n_k;
+    T t;
+    t.run(sm, A, m0, Bm, n0, k0, k1);
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+        *reinterpret_cast<float4*>(sm + t.row(i) * SC + t.col(0)) =
+            make_float4(t.c[i][0].x, t.c[i][0].y, t.c[i][1].x, t.c[i][1].y);
+    cl.sync();
+    const int rows = T::BM / ranks;
+    for (int e = threadIdx.x; e < rows * T::BN; e += 256) {
+        const int r = rank * rows + e / T::BN, x = e % T::BN;
+        const int64_t m = m0 + r, n = n0 + x;
+        if (m >= A.rows || n >= Bm.rows) continue;
+        float v = 0.f;
+        for (int j = 0; j < ranks; ++j) v += cl.map_shared_rank(sm, j)[r * SC + x];
+        if (kRelu) {
+            v += bias ? bias[n] : 0.f;
+            v = v > 0.f ? v : 0.f;
         }
+        out[m * Bm.rows + n] = v;
     }
-    if (gb1 && x == 0) gb1[f] = gs;
-    if (!gW1) return;
-    float* out = gW1 + (int64_t)f * D + x;
-    if (vec) {
-        *reinterpret_cast<float4*>(out) = acc;
+    cl.sync();  // no CTA leaves while another reads its tile
+}
+
+// dL/dW1[f, x] = sum_b g[b, f] h[b, x] and dL/db1[f] = sum_b g[b, f] (by the first x tile).
+// Either output may be NULL.
+using OuterTile = SgemmTile<8, 4, 16, false, false>;
+__global__ void __launch_bounds__(256, 2) outer_kernel(GemmSide g, GemmSide h, int64_t B, int vec,
+                                                       float* __restrict__ gW, float* __restrict__ gb) {
+    __shared__ __align__(16) float sm[OuterTile::kSmemFloats];
+    chain_launches();
+    const int64_t x0 = (int64_t)blockIdx.x * OuterTile::BN, f0 = (int64_t)blockIdx.y * OuterTile::BM;
+    OuterTile t;
+    if (x0 == 0 && gb) {
+        float db = 0.f;
+        t.template run<true>(sm, g, f0, h, x0, 0, B, &db);
+        if (threadIdx.x < OuterTile::BM && f0 + threadIdx.x < g.rows) gb[f0 + threadIdx.x] = db;
     } else {
-        out[0] = acc.x;
-        if (x + 1 < D) out[1] = acc.y;
-        if (x + 2 < D) out[2] = acc.z;
-        if (x + 3 < D) out[3] = acc.w;
+        t.run(sm, g, f0, h, x0, 0, B);
+    }
+    if (!gW) return;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int64_t f = f0 + t.row(i), x = x0 + t.col(0);
+        if (f >= g.rows) continue;
+        float* o = gW + f * h.rows + x;
+        const float4 v = make_float4(t.c[i][0].x, t.c[i][0].y, t.c[i][1].x, t.c[i][1].y);
+        if (vec && x + 4 <= h.rows) {
+            *reinterpret_cast<float4*>(o) = v;
+        } else {
+            if (x < h.rows) o[0] = v.x;
+            if (x + 1 < h.rows) o[1] = v.y;
+            if (x + 2 < h.rows) o[2] = v.z;
+            if (x + 3 < h.rows) o[3] = v.w;
+        }
     }
 }
 
-int grad_blocks(estp_ctx* ctx, int64_t total) {
-    const int64_t b = (total + 255) / 256, cap = 4 * (int64_t)ctx->num_sms;
-    return (int)(b < cap ? (b > 0 ? b : 1) : cap);
+// A matrix with `rows` rows of `n` contiguous floats: as an operand whose side is the rows
+// (k along a row) or whose side is the columns (k over the rows).
+GemmSide side_rows(const float* p, int64_t rows, int64_t n) {
+    return GemmSide{p, n, rows, n % 4 == 0 && aligned16(p) ? 1 : 0};
+}
+GemmSide side_cols(const float* p, int64_t n) { return side_rows(p, n, n); }
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch(void (*kern)(KArgs...), dim3 grid, int threads, cudaStream_t st, bool dependent, int cluster_z,
+                   Args... args) {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = st;
+    cfg.attrs = attr;
+    if (dependent) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster_z > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = 1;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = (unsigned)cluster_z;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+
+int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
+
+// Splits of a layer's contraction in logit_part_kernel: enough blocks of 32 x 32 logits to
+// occupy every SM twice, none shorter than one slice.
+struct LogitSplit {
+    int n, len;
+};
+LogitSplit logit_split(const estp_ctx* ctx, int B, int K, int64_t D) {
+    const int64_t tiles = (int64_t)ceil_div(B, LogitTile::BM) * ceil_div(K, LogitTile::BN);
+    int64_t n = 2 * ctx->num_sms / tiles;
+    n = n < 1 ? 1 : n;
+    const int64_t slices = (D + 63) / 64;
+    if (n > slices) n = slices;
+    const int64_t len = (slices + n - 1) / n * 64;
+    return LogitSplit{ceil_div(D, len), (int)len};
+}
+
+// Logits of x [B, D] through W [K, D], then the head: dz and part (training) or pred / probs.
+cudaError_t head_forward(estp_ctx* ctx, const float* x, int B, int64_t D, const float* W, const float* bias,
+                         const float* centers, int K, const float* targets, float lambda3, LogitSplit sp,
+                         float* zpart, float* dz, float2* part, float* pred, float* probs, bool dependent,
+                         cudaStream_t st) {
+    cudaError_t e = launch(logit_part_kernel,
+                           dim3((unsigned)ceil_div(B, LogitTile::BM), (unsigned)ceil_div(K, LogitTile::BN), (unsigned)sp.n),
+                           256, st, dependent, 1, side_rows(x, B, D), side_rows(W, K, D), D, sp.len, zpart);
+    if (e != cudaSuccess) return e;
+    return launch(head_loss_kernel, dim3((unsigned)B), kLossThreads, st, true, 1, (const float*)zpart, sp.n, bias, centers,
+                  K, targets, B, lambda3, dz, part, pred, probs);
+}
+
+// Gradients of that layer (grad_x gated by `gate` when given) and the loss.
+cudaError_t layer_grads(const float* x, int B, int64_t D, const float* W, int K, const float* dz,
+                        const float2* part, float lambda3, float* loss, float* grad_W, float* grad_bias,
+                        float* grad_x, const float* gate, cudaStream_t st) {
+    LayerGradArgs a{};
+    a.dz_k = side_cols(dz, K);
+    a.dz_b = side_rows(dz, B, K);
+    a.x_d = side_cols(x, D);
+    a.w_d = side_cols(W, D);
+    a.B = B; a.K = K; a.D = D;
+    a.n_wk = ceil_div(K, GradWTile::BM);
+    a.n_w = grad_W ? a.n_wk * ceil_div(D, GradWTile::BN) : grad_bias ? a.n_wk : 0;
+    a.n_x = grad_x ? ceil_div(B, GradXTile::BM) * ceil_div(D, GradXTile::BN) : 0;
+    a.grad_W = grad_W; a.grad_bias = grad_bias; a.grad_x = grad_x; a.gate = gate;
+    a.part = part; a.lambda3 = lambda3; a.loss = loss;
+    return launch(layer_grad_kernel, dim3((unsigned)(a.n_w + a.n_x + 1)), 256, st, true, 1, a);
+}
+
+// out [M, N] of wide_gemm_kernel.  The tile height follows M (a batch of prompts), so that a
+// small batch does not multiply padding; the cluster is the widest that keeps every rank two
+// slices of work and the grid within two blocks an SM.
+template <bool kAlongB, bool kRelu>
+cudaError_t wide_gemm(estp_ctx* ctx, const GemmSide& A, const GemmSide& Bm, int64_t n_k, const float* bias,
+                      float* out, bool dependent, cudaStream_t st) {
+    const int64_t M = A.rows, N = Bm.rows;
+    const int tm = M > 64 ? 8 : M > 32 ? 4 : M > 16 ? 2 : 1;
+    const dim3 tiles((unsigned)ceil_div(N, 64), (unsigned)ceil_div(M, 16 * tm));
+    int S = 8;
+    while (S > 1 && ((int64_t)tiles.x * tiles.y * S > 2 * (int64_t)ctx->num_sms || n_k / S < 128)) S /= 2;
+    const dim3 grid(tiles.x, tiles.y, (unsigned)S);
+    auto go = [&](auto kern) { return launch(kern, grid, 256, st, dependent, S, A, Bm, n_k, bias, out); };
+    return tm == 8 ? go(wide_gemm_kernel<8, 16, kAlongB, kRelu>)
+         : tm == 4 ? go(wide_gemm_kernel<4, 32, kAlongB, kRelu>)
+         : tm == 2 ? go(wide_gemm_kernel<2, 32, kAlongB, kRelu>)
+                   : go(wide_gemm_kernel<1, 64, kAlongB, kRelu>);
 }
 
 }  // namespace
@@ -329,47 +428,40 @@ estp_status launch_head_loss(estp_ctx* ctx, const float* pooled, int B, int64_t 
                              float* loss, float* grad_W, float* grad_bias, float* grad_pooled,
                              cudaStream_t st) {
     const int K = head.K;
+    const LogitSplit sp = logit_split(ctx, B, K, D);
+    // workspace: dz [B, K] | part [B] | partial logits [splits, B, K]
     const size_t off_part = align_up(sizeof(float) * (size_t)B * K, 256);
-    estp_status s = ws_reserve(ctx, off_part + sizeof(float2) * (size_t)B);
+    const size_t off_z = off_part + align_up(sizeof(float2) * (size_t)B, 256);
+    estp_status s = ws_reserve(ctx, off_z + sizeof(float) * (size_t)sp.n * B * K);
     if (s != ESTP_OK) return s;
     char* ws = static_cast<char*>(ctx->ws);
     float* dz = reinterpret_cast<float*>(ws);
     float2* part = reinterpret_cast<float2*>(ws + off_part);
-    head_fwd_kernel<<<B, kFwdThreads, 0, st>>>(pooled, D, head.W, head.bias, head.centers, K,
-                                               targets, B, lambda3, dz, part, nullptr, nullptr);
-    const int64_t total = (grad_W ? (int64_t)K * D : 0) + (grad_bias ? K : 0) +
-                          (grad_pooled ? (int64_t)B * D : 0) + 1;
-    head_grad_kernel<<<grad_blocks(ctx, total), 256, 0, st>>>(pooled, B, D, head.W, K, dz, nullptr,
-                                                              part, lambda3, loss, grad_W, grad_bias,
-                                                              grad_pooled);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = head_forward(ctx, pooled, B, D, head.W, head.bias, head.centers, K, targets, lambda3, sp,
+                                 reinterpret_cast<float*>(ws + off_z), dz, part, nullptr, nullptr, false, st);
+    if (e != cudaSuccess) return cuda_fail(e, "head forward launch");
+    e = layer_grads(pooled, B, D, head.W, K, dz, part, lambda3, loss, grad_W, grad_bias, grad_pooled, nullptr, st);
+    if (e != cudaSuccess) return cuda_fail(e, "head gradient launch");
+    e = cudaGetLastError();
     return e == cudaSuccess ? ESTP_OK : cuda_fail(e, "head loss launch");
-}
-
-// The MLP's hidden units u [B, F] into the workspace at `u`.
-static bool vec4(const float* a, const float* b, int64_t D) {
-    return D % 4 == 0 && aligned16(a) && aligned16(b);
-}
-
-static cudaError_t mlp_hidden(estp_ctx* ctx, const float* pooled, int B, int64_t D,
-                              const estp_mlp_head& head, float* u, cudaStream_t st) {
-    const int64_t threads = 32 * (int64_t)head.F;
-    mlp_hidden_kernel<<<(unsigned)((threads + 127) / 128), 128, 0, st>>>(
-        pooled, B, D, head.W1, head.b1, head.F, u, vec4(pooled, head.W1, D) ? 1 : 0);
-    return cudaGetLastError();
 }
 
 estp_status launch_mlp_head_predict(estp_ctx* ctx, const float* pooled, int B, int64_t D,
                                     const estp_mlp_head& head, float* pred, float* probs,
                                     cudaStream_t st) {
-    estp_status s = ws_reserve(ctx, sizeof(float) * (size_t)B * head.F);
+    const int F = head.F, K = head.K;
+    const LogitSplit sp = logit_split(ctx, B, K, F);
+    // workspace: u [B, F] | partial logits
+    const size_t off_z = align_up(sizeof(float) * (size_t)B * F, 256);
+    estp_status s = ws_reserve(ctx, off_z + sizeof(float) * (size_t)sp.n * B * K);
     if (s != ESTP_OK) return s;
-    float* u = static_cast<float*>(ctx->ws);
-    cudaError_t e = mlp_hidden(ctx, pooled, B, D, head, u, st);
+    char* ws = static_cast<char*>(ctx->ws);
+    float* u = reinterpret_cast<float*>(ws);
+    cudaError_t e = wide_gemm<true, true>(ctx, side_rows(pooled, B, D), side_rows(head.W1, F, D), D, head.b1, u, false, st);
     if (e != cudaSuccess) return cuda_fail(e, "mlp hidden launch");
-    head_fwd_kernel<<<B, kFwdThreads, 0, st>>>(u, head.F, head.W2, head.b2, head.centers, head.K,
-                                               nullptr, B, 0.f, nullptr, nullptr, pred, probs);
-    e = cudaGetLastError();
+    e = head_forward(ctx, u, B, F, head.W2, head.b2, head.centers, K, nullptr, 0.f, sp,
+                     reinterpret_cast<float*>(ws + off_z), nullptr, nullptr, pred, probs, true, st);
+    if (e == cudaSuccess) e = cudaGetLastError();
     return e == cudaSuccess ? ESTP_OK : cuda_fail(e, "mlp head launch");
 }
 
@@ -377,46 +469,37 @@ estp_status launch_mlp_head_loss(estp_ctx* ctx, const float* pooled, int B, int6
                                  const estp_mlp_head& head, const float* targets, float lambda3,
                                  float* loss, const estp_mlp_grads& g, cudaStream_t st) {
     const int F = head.F, K = head.K;
-    // workspace: u [B, F] | du [B, F] | dz [B, K] | part [B]
-    const size_t off_du = align_up(sizeof(float) * (size_t)B * F, 256);
-    const size_t off_dz = off_du + align_up(sizeof(float) * (size_t)B * F, 256);
+    const LogitSplit sp = logit_split(ctx, B, K, F);
+    // workspace: u [B, F] | g = dL/du where u > 0 [B, F] | dz [B, K] | part [B] | partial logits
+    const size_t off_g = align_up(sizeof(float) * (size_t)B * F, 256);
+    const size_t off_dz = 2 * off_g;
     const size_t off_part = off_dz + align_up(sizeof(float) * (size_t)B * K, 256);
-    estp_status s = ws_reserve(ctx, off_part + sizeof(float2) * (size_t)B);
+    const size_t off_z = off_part + align_up(sizeof(float2) * (size_t)B, 256);
+    estp_status s = ws_reserve(ctx, off_z + sizeof(float) * (size_t)sp.n * B * K);
     if (s != ESTP_OK) return s;
     char* ws = static_cast<char*>(ctx->ws);
     float* u = reinterpret_cast<float*>(ws);
-    float* du = reinterpret_cast<float*>(ws + off_du);
+    float* gu = reinterpret_cast<float*>(ws + off_g);
     float* dz = reinterpret_cast<float*>(ws + off_dz);
     float2* part = reinterpret_cast<float2*>(ws + off_part);
     const bool lower = g.W1 || g.b1 || g.pooled;  // gradients below the hidden layer
-    cudaError_t e = mlp_hidden(ctx, pooled, B, D, head, u, st);
+    cudaError_t e = wide_gemm<true, true>(ctx, side_rows(pooled, B, D), side_rows(head.W1, F, D), D, head.b1, u, false, st);
     if (e != cudaSuccess) return cuda_fail(e, "mlp hidden launch");
-    head_fwd_kernel<<<B, kFwdThreads, 0, st>>>(u, F, head.W2, head.b2, head.centers, K, targets, B,
-                                               lambda3, dz, part, nullptr, nullptr);
-    // second layer: dL/dW2, dL/db2, dL/du and the loss
-    int64_t total = (g.W2 ? (int64_t)K * F : 0) + (g.b2 ? K : 0) + (lower ? (int64_t)B * F : 0) + 1;
-    head_grad_kernel<<<grad_blocks(ctx, total), 256, 0, st>>>(u, B, F, head.W2, K, dz, nullptr, part,
-                                                              lambda3, loss, g.W2, g.b2,
-                                                              lower ? du : nullptr);
-    if (g.W1 || g.b1) {  // first layer, through the ReLU (u > 0): dL/dW1, dL/db1
-        const int64_t threads = (int64_t)F * ((D + 3) / 4);
-        mlp_dw1_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(
-            pooled, B, D, F, du, u, g.W1, g.b1, vec4(pooled, g.W1 ? g.W1 : pooled, D) ? 1 : 0);
+    e = head_forward(ctx, u, B, F, head.W2, head.b2, head.centers, K, targets, lambda3, sp,
+                     reinterpret_cast<float*>(ws + off_z), dz, part, nullptr, nullptr, true, st);
+    if (e != cudaSuccess) return cuda_fail(e, "mlp head launch");
+    // second layer: dL/dW2, dL/db2, dL/du through the ReLU, and the loss
+    e = layer_grads(u, B, F, head.W2, K, dz, part, lambda3, loss, g.W2, g.b2, lower ? gu : nullptr, u, st);
+    if (e != cudaSuccess) return cuda_fail(e, "mlp second-layer gradient launch");
+    if (g.W1 || g.b1) {  // first layer: dL/dW1, dL/db1
+        const GemmSide h = side_cols(pooled, D);
+        e = launch(outer_kernel, dim3((unsigned)(g.W1 ? ceil_div(D, OuterTile::BN) : 1), (unsigned)ceil_div(F, OuterTile::BM)),
+                   256, st, true, 1, side_cols(gu, F), h, (int64_t)B, h.vec && (!g.W1 || aligned16(g.W1)) ? 1 : 0, g.W1, g.b1);
+        if (e != cudaSuccess) return cuda_fail(e, "mlp first-layer gradient launch");
     }
-    const size_t smem = sizeof(float) * kDhB * (size_t)F;
-    if (g.pooled && smem > 200 * 1024) {  // very wide hidden layer: the general kernel
-        total = (int64_t)B * D;
-        head_grad_kernel<<<grad_blocks(ctx, total), 256, 0, st>>>(pooled, B, D, head.W1, F, du, u,
-                                                                  nullptr, 0.f, nullptr, nullptr,
-                                                                  nullptr, g.pooled);
-    } else if (g.pooled) {  // dL/dpooled = W1^T (dL/du where u > 0)
-        const dim3 grid((unsigned)((D + 127) / 128), (unsigned)((B + kDhB - 1) / kDhB));
-        if (smem > 48 * 1024) {
-            e = cudaFuncSetAttribute(mlp_dh_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return cuda_fail(e, "mlp input-gradient smem attribute");
-        }
-        mlp_dh_kernel<<<grid, 256, smem, st>>>(head.W1, D, F, du, u, B, g.pooled,
-                                               vec4(head.W1, head.W1, D) ? 1 : 0);
+    if (g.pooled) {  // dL/dpooled = W1^T g
+        e = wide_gemm<false, false>(ctx, side_rows(gu, B, F), side_cols(head.W1, D), F, nullptr, g.pooled, true, st);
+        if (e != cudaSuccess) return cuda_fail(e, "mlp input-gradient launch");
     }
     e = cudaGetLastError();
     return e == cudaSuccess ? ESTP_OK : cuda_fail(e, "mlp head loss launch");

@@ -5,7 +5,7 @@
 // lm_head_kernel: one persistent CTA per SM.  A work item is (row block rb of 128 tokens,
 // vocabulary split sp); items run split-fastest, so the CTAs working at one time share a
 // few row blocks (kept in L2) and stream W.  For every 256-entry vocabulary tile of its
-// split the CTA forms the 128 x 256 logit tile in TMEM,
+// split (the last one shorter, in units of 32 entries) the CTA forms the 128 x 256 logit tile in TMEM,
 //   D = sum over 64-wide chunks c of the hidden size of A_c B_c^T,
 // with A_c = hidden[rows of rb, c] and B_c = W[entries of the tile, c] staged by TMA in a
 // 4-stage ring (128B-swizzled, 48 KB per stage), 4 tcgen05.mma (M = 128, N = 256, K = 16)
@@ -17,7 +17,7 @@
 //               32-column chunks and folds them into the token's running
 //               m = max y, s = sum 2^(y - m), t = sum 2^(y - m) (y - m), y = z log2(e)
 // At the end of an item each token's (m, s, t) for the split goes to a partial buffer;
-// lm_head_merge_kernel combines the splits in split order,
+// lm_head_merge_kernel combines the splits in a fixed order,
 //   M = max m_k, S = sum 2^(m_k - M) s_k, T = sum 2^(m_k - M) (t_k + s_k (m_k - M)),
 // and writes H = ln 2 (log2 S - T / S) (nats).
 //
@@ -31,6 +31,7 @@ namespace {
 
 constexpr int kM = 128;                       // tokens per tile (TMEM lanes)
 constexpr int kN = 256;                       // vocabulary entries per tile (MMA N)
+constexpr int kUnit = 32;                     // granularity of a split and of its last tile
 constexpr int kKc = 64;                       // hidden-size chunk per stage (one swizzle atom)
 constexpr int kStages = 4;
 constexpr int kABytes = kM * kKc * 2;         // 16 KB
@@ -47,25 +48,36 @@ constexpr int kMiscOff = kBarOff + kNumBars * 8;           // tmem address, abor
 constexpr int kSmemBytes = kMiscOff + 16 + 1024;           // + alignment slack
 static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 
-// Instruction descriptor: M = 128, N = 256.
-constexpr uint32_t kIdesc = idesc_bf16(kM, kN);
-
 struct LmArgs {
     int64_t n_rows;
     int64_t V;
     int nk;            // hidden-size chunks (D / 64)
-    int n_vt;          // vocabulary tiles
+    int n_unit;        // vocabulary units of kUnit entries
     int S;             // vocabulary splits
+    int a_bytes;       // bytes of a stage's A box: 128 rows, or the rows of a single smaller block
     int64_t n_items;   // row blocks x splits
     float* part;       // [3][S][n_rows]: m, s, t (log2 units)
     int* status;
     long long wait_cycles;  // limit of the abortable waits (kWaitCycles unless a test lowers it)
 };
 
-// Vocabulary tiles [vt0, vt1) of split sp.
-__device__ __forceinline__ void split_range(const LmArgs& a, int sp, int& vt0, int& vt1) {
-    vt0 = (int)((int64_t)sp * a.n_vt / a.S);
-    vt1 = (int)((int64_t)(sp + 1) * a.n_vt / a.S);
+// Vocabulary units [u0, u1) of split sp.  Splits are cut in units and not in whole tiles, so
+// that every CTA gets the same share of W whatever V is (V = 128256 is 501 tiles, 3.3 for each of
+// 152 SMs); a split's last tile loads and multiplies only the units it has.
+__device__ __forceinline__ void split_range(const LmArgs& a, int sp, int& u0, int& u1) {
+    u0 = (int)((int64_t)sp * a.n_unit / a.S);
+    u1 = (int)((int64_t)(sp + 1) * a.n_unit / a.S);
+}
+constexpr int kTileUnits = kN / kUnit;
+
+// D (TMEM) = A B^T (+ D when acc != 0) with N = n columns.
+__device__ __forceinline__ void mma_n(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t n, uint32_t acc) {
+    const uint32_t idesc = idesc_bf16(kM, 0) | ((n >> 3) << 17);
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
 // Fold 32 logits z (one chunk of this token's row) into (m, s, t), log2 units.  Columns
@@ -112,7 +124,7 @@ __device__ __forceinline__ void fold_chunk(float* v, int valid, float& m, float&
 
 __global__ void __launch_bounds__(kThreads, 1)
     lm_head_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
-                   const LmArgs a) {
+                   const __grid_constant__ CUtensorMap tm_bu, const LmArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~uintptr_t(1023));
@@ -125,6 +137,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + kMiscOff + 4);
 
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the merge may be scheduled
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int i = 0; i < kStages; ++i) {
@@ -155,13 +168,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) {
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_a)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_b)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tm_bu)) : "memory");
             uint32_t step = 0;
             bool ok = true;
             for (int64_t item = blockIdx.x; ok && item < a.n_items; item += gridDim.x) {
                 const int sp = (int)(item % a.S), rb = (int)(item / a.S);
-                int vt0, vt1;
-                split_range(a, sp, vt0, vt1);
-                for (int vt = vt0; ok && vt < vt1; ++vt) {
+                int u0, u1;
+                split_range(a, sp, u0, u1);
+                for (int ut = u0; ok && ut < u1; ut += kTileUnits) {
+                    const int n_u = u1 - ut < kTileUnits ? u1 - ut : kTileUnits;
                     for (int kc = 0; kc < a.nk; ++kc, ++step) {
                         const int stage = (int)(step % kStages);
                         const uint32_t u = step / kStages;
@@ -170,9 +185,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                             break;
                         }
                         uint8_t* st = sm + stage * kStageBytes;
-                        mbar_expect_tx(&full[stage], kStageBytes);
+                        mbar_expect_tx(&full[stage], a.a_bytes + n_u * (kBBytes / kTileUnits));
                         tma_load_2d(st, &tm_a, kc * kKc, rb * kM, &full[stage]);
-                        tma_load_2d(st + kABytes, &tm_b, kc * kKc, vt * kN, &full[stage]);
+                        if (n_u == kTileUnits) {
+                            tma_load_2d(st + kABytes, &tm_b, kc * kKc, ut * kUnit, &full[stage]);
+                        } else {
+                            for (int j = 0; j < n_u; ++j)
+                                tma_load_2d(st + kABytes + j * (kBBytes / kTileUnits), &tm_bu, kc * kKc,
+                                            (ut + j) * kUnit, &full[stage]);
+                        }
                     }
                 }
             }
@@ -187,9 +208,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true, issued = false;
             for (int64_t item = blockIdx.x; ok && item < a.n_items; item += gridDim.x) {
                 const int sp = (int)(item % a.S);
-                int vt0, vt1;
-                split_range(a, sp, vt0, vt1);
-                for (int vt = vt0; ok && vt < vt1; ++vt, ++tile) {
+                int u0, u1;
+                split_range(a, sp, u0, u1);
+                for (int ut = u0; ok && ut < u1; ut += kTileUnits, ++tile) {
+                    const uint32_t n = (uint32_t)((u1 - ut < kTileUnits ? u1 - ut : kTileUnits) * kUnit);
                     const int ab = (int)(tile % kAccBufs);
                     const uint32_t ua = tile / kAccBufs;
                     if (ua >= 1 && !wait_bar(&acc_empty[ab], (ua - 1) & 1, abort_flag, a.status, a.wait_cycles)) {
@@ -209,8 +231,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint32_t sa = smem_u32(sm + stage * kStageBytes);
 #pragma unroll
                         for (int kk = 0; kk < kKc / 16; ++kk)
-                            mma_bf16<kIdesc>(d, sw128_desc(sa + kk * 32), sw128_desc(sa + kABytes + kk * 32),
-                                     (kc > 0 || kk > 0) ? 1u : 0u);
+                            mma_n(d, sw128_desc(sa + kk * 32), sw128_desc(sa + kABytes + kk * 32), n,
+                                  (kc > 0 || kk > 0) ? 1u : 0u);
                         mma_commit(&empty[stage]);
                     }
                     if (ok) mma_commit(&acc_full[ab]);
@@ -229,10 +251,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool ok = true;
         for (int64_t item = blockIdx.x; ok && item < a.n_items; item += gridDim.x) {
             const int sp = (int)(item % a.S), rb = (int)(item / a.S);
-            int vt0, vt1;
-            split_range(a, sp, vt0, vt1);
+            int u0, u1;
+            split_range(a, sp, u0, u1);
             float m = -INFINITY, s = 0.f, t = 0.f;
-            for (int vt = vt0; vt < vt1; ++vt, ++tile) {
+            for (int ut = u0; ut < u1; ut += kTileUnits, ++tile) {
+                const int n_u = u1 - ut < kTileUnits ? u1 - ut : kTileUnits;
                 const int ab = (int)(tile % kAccBufs);
                 if (!warp_wait(&acc_full[ab], (tile / kAccBufs) & 1, abort_flag, a.status, a.wait_cycles)) {
                     ok = false;
@@ -240,19 +263,18 @@ __global__ void __launch_bounds__(kThreads, 1)
                 }
                 tc_fence_after();
                 const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(ab * kN);
-                const int64_t v0 = (int64_t)vt * kN;
+                const int64_t v0 = (int64_t)ut * kUnit;
 #pragma unroll 1
-                for (int ch = 0; ch < kN / 32; ++ch) {
+                for (int ch = 0; ch < n_u; ++ch) {  // a unit is one 32-column load
                     float v[32];
                     tmem_ld32(taddr + ch * 32, v);
                     tmem_wait_ld();
-                    if (ch == kN / 32 - 1) {  // the whole tile is in registers: release it
+                    if (ch == n_u - 1) {  // the whole tile is in registers: release it
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&acc_empty[ab]);
                     }
                     const int64_t left = a.V - (v0 + ch * 32);
-                    if (left <= 0) continue;
                     fold_chunk(v, left < 32 ? (int)left : 32, m, s, t);
                 }
             }
@@ -277,23 +299,53 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
-// Per token: the splits' (m, s, t) combined in split order, H in nats.
-__global__ void lm_head_merge_kernel(const float* __restrict__ part, int64_t n_rows, int S,
-                                     float* __restrict__ H) {
-    const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rows) return;
+// Per token: the splits' (m, s, t) combined, H in nats.  A block takes 32 tokens; its warp y the
+// splits y, y + Y, .. of each in order, and the Y results are combined in warp order (a fixed
+// order, whatever the launch).  A small batch has as many splits as vocabulary tiles (594 for 37
+// tokens of a 152064-entry vocabulary), which one thread a token read one after another: 198 us there
+// (the call 342 us, against 176 now).  Launched as a programmatic dependent of lm_head_kernel.
+constexpr int kMergeWarps = 32;
+__device__ __forceinline__ void merge_split(float& M, float& S, float& T, float m, float s, float t) {
+    const float mm = fmaxf(M, m);
+    if (mm == -INFINITY) return;  // splits without vocabulary entries
+    const float da = M - mm, db = m - mm;
+    // an empty side (-inf) has S = T = 0 and a weight of 0
+    const float fa = M == -INFINITY ? 0.f : ex2(da), fb = m == -INFINITY ? 0.f : ex2(db);
+    T = (M == -INFINITY ? 0.f : fa * fmaf(S, da, T)) + (m == -INFINITY ? 0.f : fb * fmaf(s, db, t));
+    S = fa * S + fb * s;
+    M = mm;
+}
+
+__global__ void __launch_bounds__(32 * kMergeWarps) lm_head_merge_kernel(const float* part, int64_t n_rows, int S,
+                                                                          float* __restrict__ H) {
+    __shared__ float3 red[kMergeWarps][32];
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the partials are complete
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    const int64_t r = (int64_t)blockIdx.x * 32 + lane;
     const int64_t plane = (int64_t)S * n_rows;
-    float M = -INFINITY;
-    for (int k = 0; k < S; ++k) M = fmaxf(M, part[(int64_t)k * n_rows + r]);
-    float Sx = 0.f, Tx = 0.f;
-    for (int k = 0; k < S; ++k) {
-        const float mk = part[(int64_t)k * n_rows + r];
-        const float sk = part[plane + (int64_t)k * n_rows + r];
-        const float tk = part[2 * plane + (int64_t)k * n_rows + r];
-        if (mk == -INFINITY) continue;  // a split without vocabulary entries
-        const float dm = mk - M, f = ex2(dm);
-        Sx = fmaf(f, sk, Sx);
-        Tx = fmaf(f, fmaf(sk, dm, tk), Tx);
+    float M = -INFINITY, Sx = 0.f, Tx = 0.f;
+    if (r < n_rows) {
+        constexpr int kBatch = 4;  // splits whose loads are in flight at once
+        for (int k0 = warp; k0 < S; k0 += kBatch * n_warps) {
+            float m[kBatch], s[kBatch], t[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                const int k = k0 + j * n_warps;
+                const float* p = part + (int64_t)k * n_rows + r;
+                m[j] = k < S ? p[0] : -INFINITY;
+                s[j] = k < S ? p[plane] : 0.f;
+                t[j] = k < S ? p[2 * plane] : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) merge_split(M, Sx, Tx, m[j], s[j], t[j]);
+        }
+    }
+    red[warp][lane] = make_float3(M, Sx, Tx);
+    __syncthreads();
+    if (warp != 0 || r >= n_rows) return;
+    for (int w = 1; w < n_warps; ++w) {
+        const float3 o = red[w][lane];
+        merge_split(M, Sx, Tx, o.x, o.y, o.z);
     }
     H[r] = kLn2 * (lg2(Sx) - Tx / Sx);
 }
@@ -321,31 +373,38 @@ estp_status make_map_2d(CUtensorMap* m, const void* base, int64_t D, int64_t row
 estp_status launch_lm_head_entropy(estp_ctx* ctx, const void* hidden, int64_t ldh, const void* W,
                                    int64_t ldw, int64_t n_rows, int64_t D, int64_t V, float* H,
                                    cudaStream_t st) {
-    CUtensorMap tma, tmb;
-    estp_status s = make_map_2d(&tma, hidden, D, n_rows, ldh, kM);
+    CUtensorMap tma, tmb, tmbu;
+    // a batch of fewer rows than a tile loads only those (in groups of 8): what the other rows of
+    // the shared tile hold goes to logits that no one reads.  (A box of 128 rows around one row of a
+    // 4096-wide hidden state: the call 220 us against 173.)
+    const int a_rows = n_rows < kM ? (int)(n_rows + 7) / 8 * 8 : kM;
+    estp_status s = make_map_2d(&tma, hidden, D, n_rows, ldh, a_rows);
     if (s != ESTP_OK) return s;
     s = make_map_2d(&tmb, W, D, V, ldw, kN);
+    if (s != ESTP_OK) return s;
+    s = make_map_2d(&tmbu, W, D, V, ldw, kUnit);
     if (s != ESTP_OK) return s;
     LmArgs a{};
     a.n_rows = n_rows;
     a.V = V;
     a.nk = (int)(D / kKc);
-    a.n_vt = (int)((V + kN - 1) / kN);
+    a.n_unit = (int)((V + kUnit - 1) / kUnit);
     const int64_t n_rb = (n_rows + kM - 1) / kM;
-    // splits: at least four items per SM; the fewest splits whose items fill the last
-    // wave of the persistent grid to 97 % (else the best fill up to four times as many).
-    // Fewer splits keep more row blocks in flight at once, so that each W tile read from
-    // DRAM serves more of them.
+    // splits: the fewest whose items fill the last wave of the persistent grid to 97 % (else
+    // the best fill up to four times as many).  Fewer splits keep more row blocks in flight at
+    // once, so that each W tile read from DRAM serves more of them.  (Cut in units of 32 entries the
+    // splits are equal, so one item an SM is enough: at least four, cut in whole tiles, took 3026 us
+    // for 4103 x 4096 x 128256 against 2731, 604 against 512 for 1291 x 3776 x 68767.)
     // At least as many splits that the row blocks in flight at once (G / S of them, 256 D
     // bytes each) fit in ~48 MB of L2 beside the W tiles streaming through.
     const int64_t G = ctx->num_sms;
     const int64_t l2_budget = 48ll << 20, rb_bytes = (int64_t)kM * D * 2;
     const int64_t s_l2 = (G * rb_bytes + l2_budget - 1) / l2_budget;
-    int64_t s_lo = (4 * G + n_rb - 1) / n_rb;
+    int64_t s_lo = G / n_rb > 0 ? G / n_rb : 1;
     if (s_lo < s_l2) s_lo = s_l2;
-    int64_t S = s_lo < a.n_vt ? s_lo : a.n_vt;  // small problems: one tile per split
+    int64_t S = s_lo < a.n_unit ? s_lo : a.n_unit;  // small problems: one unit per split
     double best = -1.0;
-    for (int64_t c = s_lo; c <= a.n_vt && c <= 4 * s_lo; ++c) {
+    for (int64_t c = s_lo; c <= a.n_unit && c <= 4 * s_lo; ++c) {
         const int64_t items = n_rb * c, waves = (items + G - 1) / G;
         const double fill = (double)items / (double)(waves * G);
         if (fill > best + 1e-9) {
@@ -355,6 +414,7 @@ estp_status launch_lm_head_entropy(estp_ctx* ctx, const void* hidden, int64_t ld
         if (fill >= 0.97) break;
     }
     a.S = (int)S;
+    a.a_bytes = a_rows * kKc * 2;
     a.n_items = n_rb * S;
     s = ws_reserve(ctx, sizeof(float) * 3 * (size_t)S * (size_t)n_rows);
     if (s != ESTP_OK) return s;
@@ -365,11 +425,22 @@ estp_status launch_lm_head_entropy(estp_ctx* ctx, const void* hidden, int64_t ld
                                          kSmemBytes);
     if (e != cudaSuccess) return cuda_fail(e, "lm-head kernel smem attribute");
     const int64_t grid = a.n_items < ctx->num_sms ? a.n_items : ctx->num_sms;
-    lm_head_kernel<<<(unsigned)grid, kThreads, kSmemBytes, st>>>(tma, tmb, a);
+    lm_head_kernel<<<(unsigned)grid, kThreads, kSmemBytes, st>>>(tma, tmb, tmbu, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "lm-head kernel launch");
-    lm_head_merge_kernel<<<(unsigned)((n_rows + 255) / 256), 256, 0, st>>>(a.part, n_rows, a.S, H);
-    e = cudaGetLastError();
+    // a warp per four splits (the merge's batch), at most kMergeWarps
+    const int mw = a.S >= 4 * kMergeWarps ? kMergeWarps : (a.S + 3) / 4;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n_rows + 31) / 32));
+    cfg.blockDim = dim3((unsigned)(32 * mw));
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, lm_head_merge_kernel, (const float*)a.part, n_rows, a.S, H);
+    if (e == cudaSuccess) e = cudaGetLastError();
     return e == cudaSuccess ? ESTP_OK : cuda_fail(e, "lm-head merge launch");
 }
 

@@ -9,8 +9,11 @@
 // A_ij = 2^(s_ij log2e - lse_i log2e) stays in the thread that owns key j.  Each
 // item writes its keys' partial sums to its own slot of a partial buffer; the reduce
 // kernel adds the slots of every key in a fixed order (no float atomics).
+#include <type_traits>
+
 #include "importance_plan.cuh"
 #include "importance_tc.cuh"
+#include "sgemm.cuh"
 
 namespace estp {
 
@@ -94,126 +97,112 @@ __global__ void __launch_bounds__(1024) attn_plan2_kernel(const int32_t* cu, int
 namespace {
 
 // ----------------------------------------------------------- CUDA-core kernels
-constexpr int kSTile = 64;      // rows per tile (keys or queries)
-constexpr int kSQc = 8;         // query tiles per importance item
-constexpr int kSThreads = 256;  // 16 x 16 threads, 4 x 4 scores each
+// fp32 inputs: the scores are formed on the FMA pipe (the tensor cores take no fp32 operands)
+// in the register tiles of sgemm.cuh.  An item's fixed side is kRows = 16 TM rows (128, or 64
+// where 128 would leave SMs idle), its streamed side comes in tiles of 128, and whatever of a
+// tile is wholly masked (above the diagonal, past the prompt) is left out in units of 64.
+// The bound is the FMA pipe (54 packed FMAs a clock and SM): a 128 x 128 tile takes 32 packed
+// FMAs a thread for four 16-byte shared loads.  Items come from a counter, the longest of a
+// prompt first.  4 prompts of 300 to 1500 tokens, 16 heads, d 128: row normalisers 485 -> 173 us,
+// column sums 857 -> 162 us against 64 x 64 tiles of scalar FMAs (4 x 4 a thread).
+constexpr int kFThreads = 256;
+constexpr int kFCols = 128;          // rows of a streamed tile
+// Items per SM below which the split gets finer.  Row normalisers at 3.2 items of 128 rows per
+// SM: 173 us with 128 rows, 183 with 64.  Column sums there: 243 us at 2 items per SM, 162 at 4
+// or 8, 234 at 16.
+constexpr int kFLseItemsPerSm = 3, kFImpItemsPerSm = 4;
 
-struct SimtArgs {
-    const void* Q;
-    const void* K;
-    const float* lse;          // [Hq, sumT] natural log
+template <int TM, int TN>
+using ScoreTile = SgemmTile<TM, TN, 16, true, true, false>;
+constexpr int kFSmem = ScoreTile<8, 8>::kSmemFloats;
+
+struct F32Args {
+    const float* Q;
+    const float* K;
+    const float* lse;          // column sums: [Hq, sumT] natural log
     const int32_t* cu;
     const int32_t* base;
-    const PlanInfo* info;
+    PlanInfo* info;
     int B, Hq, Hkv, d;
     int64_t sumT;
     float scale_log2;          // softmax_scale * log2(e)
     ImpHeads hs;
     int exclude_self;
-    float* part;               // [c_max][n_groups][sumT]
-    float* lse_out;            // LSE kernel output [Hq, sumT]
+    int qc;                    // column sums: query tiles per item
+    float* part;               // column sums: [c_max][n_groups][sumT]
+    float* lse_out;            // row normalisers: [Hq, sumT]
     int c_max;                 // chunk slots of part (bounds checks of debug builds)
     int* status;
 };
 
-// Rows [row0, row0 + n) of a [rows, heads, d] tensor, head h, into smem as fp32
-// row-major with stride d + 4; rows past n are zero.
-template <bool kBf16>
-__device__ __forceinline__ void load_tile(float* sm, const void* src, int64_t row0, int n,
-                                          int heads, int h, int d) {
-    const int stride = d + 4;
-    const int vec = kBf16 ? 8 : 4;
-    const int per_row = d / vec;
-    for (int idx = threadIdx.x; idx < kSTile * per_row; idx += kSThreads) {
-        const int r = idx / per_row, x = (idx - r * per_row) * vec;
-        float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-        if (r < n) {
-            const int64_t off = ((row0 + r) * heads + h) * (int64_t)d + x;
-            if (kBf16) {
-                uint4 v = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(src) + off);
-                lo = make_float4(bf16lo(v.x), bf16hi(v.x), bf16lo(v.y), bf16hi(v.y));
-                hi = make_float4(bf16lo(v.z), bf16hi(v.z), bf16lo(v.w), bf16hi(v.w));
-            } else {
-                lo = *reinterpret_cast<const float4*>(static_cast<const float*>(src) + off);
-            }
-        }
-        *reinterpret_cast<float4*>(sm + r * stride + x) = lo;
-        if (kBf16) *reinterpret_cast<float4*>(sm + r * stride + x + 4) = hi;
-    }
+// Items of a block: its own index first, then the plan's counter.
+__device__ __forceinline__ int next_item(PlanInfo* info, int* slot) {
+    __syncthreads();
+    if (threadIdx.x == 0) *slot = (int)gridDim.x + atomicAdd(&info->next, 1);
+    __syncthreads();
+    return *slot;
 }
 
-// acc[a][b] = A-row (ty*4+a) . B-row (tx*4+b)
-__device__ __forceinline__ void tile_dot(const float* As, const float* Bs, int d, int ty, int tx,
-                                         float acc[4][4]) {
-    const int stride = d + 4;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-    for (int x = 0; x < d; x += 4) {
-        float4 av[4], bv[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) av[a] = *reinterpret_cast<const float4*>(As + (ty * 4 + a) * stride + x);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) bv[b] = *reinterpret_cast<const float4*>(Bs + (tx * 4 + b) * stride + x);
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                acc[a][b] = fmaf(av[a].x, bv[b].x, acc[a][b]);
-                acc[a][b] = fmaf(av[a].y, bv[b].y, acc[a][b]);
-                acc[a][b] = fmaf(av[a].z, bv[b].z, acc[a][b]);
-                acc[a][b] = fmaf(av[a].w, bv[b].w, acc[a][b]);
-            }
-    }
-}
-
-// Row log-normalisers: rows = queries of one tile, streamed over key tiles 0..qt.
-template <bool kBf16>
-__global__ void __launch_bounds__(kSThreads) lse_simt_kernel(SimtArgs a) {
-    extern __shared__ float smem[];
-    float* Qs = smem;
-    float* Ks = smem + kSTile * (a.d + 4);
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+// Row log-normalisers: rows = queries of one tile, streamed over the keys up to its diagonal.
+template <int TM>
+__global__ void __launch_bounds__(kFThreads, TM == 8 ? 1 : 2) lse_f32_kernel(const F32Args a) {
+    __shared__ __align__(16) float sm[kFSmem];
+    __shared__ int slot;
+    constexpr int kRows = 16 * TM;
     const int total = a.info->total;
     const int rep = a.Hq / a.Hkv;
-    for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const LseItem it = decode_lse_item(item, a.base, a.B, a.cu, kSTile, a.hs.n_heads);
+    for (int item = blockIdx.x; item < total; item = next_item(a.info, &slot)) {
+        const LseItem it = decode_lse_item(item, a.base, a.B, a.cu, kRows, a.hs.n_heads);
         const int h = a.hs.head_list[it.hslot];
-        const int q0 = it.qt * kSTile;
-        __syncthreads();
-        load_tile<kBf16>(Qs, a.Q, it.t0 + q0, min(kSTile, it.T - q0), a.Hq, h, a.d);
-        float m[4], s[4];
+        const int q0 = it.qt * kRows;
+        const GemmSide qs{a.Q + (it.t0 * a.Hq + h) * a.d, (int64_t)a.Hq * a.d, it.T, 1};
+        const GemmSide ks{a.K + (it.t0 * a.Hkv + h / rep) * a.d, (int64_t)a.Hkv * a.d, it.T, 1};
+        float m[TM], s[TM];
 #pragma unroll
-        for (int r = 0; r < 4; ++r) { m[r] = -1e30f; s[r] = 0.f; }
-        for (int kt = 0; kt <= it.qt; ++kt) {
-            const int k0 = kt * kSTile;
-            __syncthreads();
-            load_tile<kBf16>(Ks, a.K, it.t0 + k0, min(kSTile, it.T - k0), a.Hkv, h / rep, a.d);
-            __syncthreads();
-            float acc[4][4];
-            tile_dot(Qs, Ks, a.d, ty, tx, acc);
+        for (int r = 0; r < TM; ++r) { m[r] = -1e30f; s[r] = 0.f; }
+        // rows q0 + r0 .. of R x 16 rows against C x 16 keys from k0
+        auto tile = [&](auto R, auto C, auto r0c, int k0) {
+            constexpr int kR = decltype(R)::value, kC = decltype(C)::value, r0 = decltype(r0c)::value;
+            using Tile = ScoreTile<kR, kC>;
+            Tile t;
+            t.run(sm, qs, q0 + r0, ks, k0, 0, a.d);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int i = q0 + ty * 4 + r;
-                float v[4];
+            for (int r = 0; r < kR; ++r) {
+                const int i = q0 + r0 + Tile::row(r);
+                float v[kC];
                 float mx = -1e30f;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int j = k0 + tx * 4 + c;
-                    const bool ok = j <= i && j < it.T;
-                    v[c] = ok ? acc[r][c] * a.scale_log2 : -1e30f;
+                for (int c = 0; c < kC; ++c) {
+                    const int j = k0 + Tile::col(c);
+                    const float x = c & 1 ? t.c[r][c >> 1].y : t.c[r][c >> 1].x;
+                    v[c] = j <= i && j < it.T ? x * a.scale_log2 : -1e30f;
                     mx = fmaxf(mx, v[c]);
                 }
-                const float nm = fmaxf(m[r], mx);
-                s[r] *= ex2(m[r] - nm);
-                m[r] = nm;
+                float& mr = m[r0 / 16 + r];
+                float& sr = s[r0 / 16 + r];
+                const float nm = fmaxf(mr, mx);
+                sr *= ex2(mr - nm);
+                mr = nm;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) s[r] += ex2(v[c] - nm);
+                for (int c = 0; c < kC; ++c) sr += ex2(v[c] - nm);
             }
+        };
+        using std::integral_constant;
+        constexpr integral_constant<int, 8> c8{};
+        constexpr integral_constant<int, 4> c4{};
+        constexpr integral_constant<int, 0> z{};
+        if (TM == 8 && it.T - q0 > 64) {
+            constexpr integral_constant<int, TM> full{};
+            for (int k0 = 0; k0 < q0; k0 += kFCols) tile(full, c8, z, k0);
+            tile(full, c4, z, q0);  // diagonal: 64 keys for all rows, the next 64 for the lower half
+            if constexpr (TM == 8) tile(c4, c4, integral_constant<int, 64>{}, q0 + 64);
+        } else {  // 64 rows
+            int k0 = 0;
+            for (; k0 + kFCols <= q0; k0 += kFCols) tile(c4, c8, z, k0);
+            for (; k0 <= q0; k0 += 64) tile(c4, c4, z, k0);
         }
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
+        for (int r = 0; r < TM; ++r) {
 #pragma unroll
             for (int off = 8; off > 0; off >>= 1) {
                 const float m2 = __shfl_xor_sync(0xffffffffu, m[r], off);
@@ -222,68 +211,89 @@ __global__ void __launch_bounds__(kSThreads) lse_simt_kernel(SimtArgs a) {
                 s[r] = s[r] * ex2(m[r] - nm) + s2 * ex2(m2 - nm);
                 m[r] = nm;
             }
-            const int i = q0 + ty * 4 + r;
-            if (tx == 0 && i < it.T) a.lse_out[(int64_t)h * a.sumT + it.t0 + i] = (m[r] + lg2(s[r])) * kLn2;
+            const int i = q0 + ScoreTile<TM, 4>::row(r);
+            if ((threadIdx.x & 15) == 0 && i < it.T)
+                a.lse_out[(int64_t)h * a.sumT + it.t0 + i] = (m[r] + lg2(s[r])) * kLn2;
         }
     }
 }
 
-// Column sums: rows = keys of one tile, streamed over the item's query tiles and
-// the selected heads of one KV group.
-template <bool kBf16>
-__global__ void __launch_bounds__(kSThreads) imp_simt_kernel(SimtArgs a) {
-    extern __shared__ float smem[];
-    float* Ks = smem;
-    float* Qs = smem + kSTile * (a.d + 4);
-    float* lse_s = Qs + kSTile * (a.d + 4);
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+// Column sums: rows = keys of one tile, streamed over the item's queries and heads.
+template <int TM>
+__global__ void __launch_bounds__(kFThreads, 2) imp_f32_kernel(const F32Args a) {
+    __shared__ __align__(16) float sm[kFSmem];
+    __shared__ int slot;
+    constexpr int kRows = 16 * TM;
     const int total = a.info->total;
-    for (int item = blockIdx.x; item < total; item += gridDim.x) {
-        const ImpItem it = decode_imp_item(item, a.base, a.B, a.cu, kSTile, kSQc);
-        const int grp = a.hs.group[it.g];
-        const int k0 = it.kt * kSTile;
-        __syncthreads();
-        load_tile<kBf16>(Ks, a.K, it.t0 + k0, min(kSTile, it.T - k0), a.Hkv, grp, a.d);
-        float col[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int item = blockIdx.x; item < total; item = next_item(a.info, &slot)) {
+        const ImpItem it = decode_imp_item(item, a.base, a.B, a.cu, kRows, a.qc);
+        const int k0 = it.kt * kRows;
+        const int i_end = min(it.T, it.qt1 * kRows);  // queries of the item
+        const GemmSide ks{a.K + (it.t0 * a.Hkv + a.hs.group[it.g]) * a.d, (int64_t)a.Hkv * a.d, it.T, 1};
+        float col[TM];
+#pragma unroll
+        for (int r = 0; r < TM; ++r) col[r] = 0.f;
         for (int hi = a.hs.begin[it.g]; hi < a.hs.begin[it.g + 1]; ++hi) {
             const int h = a.hs.head_list[hi];
-            for (int qt = it.qt0; qt < it.qt1; ++qt) {
-                const int q0 = qt * kSTile;
-                __syncthreads();
-                load_tile<kBf16>(Qs, a.Q, it.t0 + q0, min(kSTile, it.T - q0), a.Hq, h, a.d);
-                if (threadIdx.x < kSTile) {
-                    const int i = q0 + threadIdx.x;
-                    lse_s[threadIdx.x] = i < it.T ? a.lse[(int64_t)h * a.sumT + it.t0 + i] * kLog2e : INFINITY;
+            const GemmSide qs{a.Q + (it.t0 * a.Hq + h) * a.d, (int64_t)a.Hq * a.d, it.T, 1};
+            const float* lse = a.lse + (int64_t)h * a.sumT + it.t0;
+            // keys k0 .. of R x 16 keys against C x 16 queries from i0
+            auto tile = [&](auto R, auto C, int i0) {
+                constexpr int kR = decltype(R)::value, kC = decltype(C)::value;
+                using Tile = ScoreTile<kR, kC>;
+                Tile t;
+                t.run(sm, ks, k0, qs, i0, 0, a.d);
+                float nl[kC];  // -lse log2e
+#pragma unroll
+                for (int c = 0; c < kC; ++c) {
+                    const int i = i0 + Tile::col(c);
+                    nl[c] = i < it.T ? -lse[i] * kLog2e : -INFINITY;
                 }
-                __syncthreads();
-                float acc[4][4];
-                tile_dot(Ks, Qs, a.d, ty, tx, acc);
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int j = k0 + ty * 4 + r;
+                for (int r = 0; r < kR; ++r) {
+                    const int j = k0 + Tile::row(r);
+                    float v = 0.f;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int i = q0 + tx * 4 + c;
-                        const bool ok = i >= j && i < it.T && !(a.exclude_self && i == j);
-                        col[r] += ok ? ex2(acc[r][c] * a.scale_log2 - lse_s[tx * 4 + c]) : 0.f;
+                    for (int c = 0; c < kC; ++c) {
+                        const int i = i0 + Tile::col(c);
+                        const float x = c & 1 ? t.c[r][c >> 1].y : t.c[r][c >> 1].x;
+                        const bool ok = i >= j + a.exclude_self && i < it.T;
+                        v += ok ? ex2(fmaf(x, a.scale_log2, nl[c])) : 0.f;
                     }
+                    col[r] += v;
                 }
+            };
+            constexpr std::integral_constant<int, 8> c8{};
+            constexpr std::integral_constant<int, 4> c4{};
+            int i0 = it.qt0 * kRows;
+            if (TM == 8 && it.T - k0 > 64) {
+                constexpr std::integral_constant<int, TM> full{};
+                if (i0 == k0) {  // diagonal: the first 64 queries see the first 64 keys only
+                    tile(c4, c4, i0);
+                    tile(full, c4, i0 + 64);
+                    i0 += 128;
+                }
+                for (; i0 + 64 < i_end; i0 += kFCols) tile(full, c8, i0);
+                if (i0 < i_end) tile(full, c4, i0);
+            } else {  // 64 keys
+                for (; i0 + 64 < i_end; i0 += kFCols) tile(c4, c8, i0);
+                if (i0 < i_end) tile(c4, c4, i0);
             }
         }
-        const int c_slot = (it.qt0 - it.kt) / kSQc;
+        const int c_slot = (it.qt0 - it.kt) / a.qc;
         if (!in_bounds(c_slot >= 0 && c_slot < a.c_max, a.status)) continue;
         float* out = a.part + ((int64_t)c_slot * a.hs.n_groups + it.g) * a.sumT + it.t0;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
+        for (int r = 0; r < TM; ++r) {
 #pragma unroll
             for (int off = 8; off > 0; off >>= 1) col[r] += __shfl_xor_sync(0xffffffffu, col[r], off);
-            const int j = k0 + ty * 4 + r;
-            if (tx == 0 && j < it.T) out[j] = col[r];
+            const int j = k0 + ScoreTile<TM, 4>::row(r);
+            if ((threadIdx.x & 15) == 0 && j < it.T) out[j] = col[r];
         }
     }
 }
 
-// acc[j] (+)= sum over chunk slots c (in order) and group slots g (in order) of part.
+// acc[j] (+)= sum over chunk slots c and group slots g of part, in a fixed order.
 // Largest b with cu[b] <= j: cu staged in shared memory when it fits (kCuStage entries).
 constexpr int kCuStage = 2048;
 
@@ -312,16 +322,18 @@ __global__ void imp_reduce_kernel(const float* part, const PlanInfo* info, const
         const int kt = (int)((j - cuv[b]) / tile);
         int n = chunks_of(nt, kt, qc) * n_groups;  // partials (c, g), c-major
         if (!in_bounds(n <= c_max * n_groups && b >= 0 && b < B, status)) n = 0;
-        // up to 16 partials are loaded before any is added (independent loads in flight),
-        // then added in the same (c, g) order
+        // up to 16 partials are loaded before any is added (independent loads in flight), then
+        // added as a tree, so that a sum of n partials has chains of n / 16 additions
         constexpr int kBatch = 16;
         for (int i0 = 0; i0 < n; i0 += kBatch) {
             float p[kBatch];
 #pragma unroll
             for (int i = 0; i < kBatch; ++i) p[i] = i0 + i < n ? part[(int64_t)(i0 + i) * sumT + j] : 0.f;
 #pragma unroll
-            for (int i = 0; i < kBatch; ++i)
-                if (i0 + i < n) v += p[i];
+            for (int w = kBatch / 2; w > 0; w >>= 1)
+#pragma unroll
+                for (int i = 0; i < w; ++i) p[i] += p[i + w];
+            v += p[0];
         }
     }
     acc[j] = accumulate ? acc[j] + v : v;
@@ -344,18 +356,78 @@ __global__ void imp_finalize_kernel(const float* acc, const int32_t* cu, int B, 
     out[j] = n > 0 ? acc[j] * inv_lh / (float)n : 0.f;
 }
 
-size_t simt_smem(int d, bool with_lse) {
-    return sizeof(float) * (2 * kSTile * (d + 4) + (with_lse ? kSTile : 0));
+// Rows of an fp32 item's fixed side, query tiles per column-sum item, and whether each head
+// gets column-sum items of its own (else a KV group's heads share them).
+struct F32Split {
+    int rows, qc;
+    bool per_head;
+};
+
+// Tiles of a prompt of mean length: the lengths themselves stay on the device.
+int64_t mean_tiles(int B, int64_t sumT, int rows) {
+    const int64_t t = B > 0 ? (sumT + B - 1) / B : 0;
+    return (t + rows - 1) / rows;
+}
+
+int f32_rows(int B, int64_t sumT, int n_heads, int num_sms) {
+    return (int64_t)B * n_heads * mean_tiles(B, sumT, 128) >= (int64_t)kFLseItemsPerSm * num_sms ? 128 : 64;
+}
+
+F32Split f32_split(int B, int64_t sumT, const ImpHeads& hs, int num_sms) {
+    F32Split s{128, 8, false};
+    auto enough = [&] {
+        const int64_t lists = (int64_t)B * (s.per_head ? hs.n_heads : hs.n_groups);
+        return lists * items_f(mean_tiles(B, sumT, s.rows), s.qc) >= (int64_t)kFImpItemsPerSm * num_sms;
+    };
+    if (!enough()) s.per_head = true;
+    while (!enough() && s.qc > 1) s.qc /= 2;
+    if (!enough()) s.rows = 64;
+    return s;
+}
+
+// A group of its own for every head.
+ImpHeads heads_apart(const ImpHeads& hs, int rep) {
+    ImpHeads o = hs;
+    o.n_groups = hs.n_heads;
+    for (int i = 0; i < hs.n_heads; ++i) {
+        o.group[i] = (int16_t)(hs.head_list[i] / rep);
+        o.begin[i] = (int16_t)i;
+    }
+    o.begin[hs.n_heads] = (int16_t)hs.n_heads;
+    return o;
+}
+
+template <class Kernel>
+cudaError_t launch_f32(estp_ctx* ctx, Kernel kernel, const F32Args& a, cudaStream_t st) {
+    int occ = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kFThreads, 0);
+    if (e != cudaSuccess) return e;
+    kernel<<<ctx->num_sms * (occ > 0 ? occ : 1), kFThreads, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+// Row normalisers of the selected heads (fp32), with the plan at byte ws_off of the workspace.
+estp_status launch_lse_f32(estp_ctx* ctx, const void* Q, const void* K, int Hq, int Hkv, int d,
+                           float scale, const ImpHeads& hs, const int32_t* cu, int B, int64_t sumT,
+                           int max_seqlen, float* lse, cudaStream_t st, size_t ws_off) {
+    char* ws = static_cast<char*>(ctx->ws) + ws_off;
+    F32Args a{};
+    a.Q = static_cast<const float*>(Q); a.K = static_cast<const float*>(K);
+    a.cu = cu; a.B = B; a.Hq = Hq; a.Hkv = Hkv; a.d = d; a.sumT = sumT;
+    a.info = reinterpret_cast<PlanInfo*>(ws + align_up(sizeof(int32_t) * (size_t)(B + 1), 256));
+    a.base = reinterpret_cast<int32_t*>(ws);
+    a.scale_log2 = scale * kLog2e;
+    a.hs = hs;
+    a.lse_out = lse;
+    const int rows = f32_rows(B, sumT, hs.n_heads, ctx->num_sms);
+    attn_plan_kernel<<<1, 1024, 0, st>>>(cu, B, sumT, max_seqlen, rows, 1, hs.n_heads, 1,
+                                         reinterpret_cast<int32_t*>(ws), a.info, ctx->status);
+    const cudaError_t e = rows == 128 ? launch_f32(ctx, lse_f32_kernel<8>, a, st)
+                                      : launch_f32(ctx, lse_f32_kernel<4>, a, st);
+    return e == cudaSuccess ? ESTP_OK : cuda_fail(e, "lse launch");
 }
 
 }  // namespace
-
-// Launch geometry shared by both paths.
-static int persistent_grid(estp_ctx* ctx, const void* kernel, int threads, size_t smem) {
-    int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem);
-    return ctx->num_sms * (occ > 0 ? occ : 1);
-}
 
 estp_status launch_lse(estp_ctx* ctx, const void* Q, const void* K, estp_dtype dtype, int Hq,
                        int Hkv, int d, float scale, const ImpHeads& hs, const int32_t* cu,
@@ -365,35 +437,20 @@ estp_status launch_lse(estp_ctx* ctx, const void* Q, const void* K, estp_dtype d
     const size_t off_info = align_up(sizeof(int32_t) * (size_t)(B + 1), 256);
     estp_status s = ws_reserve(ctx, off_info + sizeof(PlanInfo));
     if (s != ESTP_OK) return s;
-    char* ws = static_cast<char*>(ctx->ws);
-    SimtArgs a{};
-    a.Q = Q; a.K = K; a.cu = cu; a.B = B; a.Hq = Hq; a.Hkv = Hkv; a.d = d; a.sumT = sumT;
-    a.base = reinterpret_cast<int32_t*>(ws);
-    a.info = reinterpret_cast<PlanInfo*>(ws + off_info);
-    a.scale_log2 = scale * kLog2e;
-    a.hs = hs;
-    a.lse_out = lse;
-    attn_plan_kernel<<<1, 1024, 0, st>>>(cu, B, sumT, max_seqlen, kSTile, 1, hs.n_heads, 1,
-                                         reinterpret_cast<int32_t*>(ws),
-                                         reinterpret_cast<PlanInfo*>(ws + off_info), ctx->status);
-    const size_t smem = simt_smem(d, false);
-    const void* kfn = dtype == ESTP_BF16 ? (const void*)lse_simt_kernel<true> : (const void*)lse_simt_kernel<false>;
-    cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    const int grid = persistent_grid(ctx, kfn, kSThreads, smem);
-    if (dtype == ESTP_BF16) lse_simt_kernel<true><<<grid, kSThreads, smem, st>>>(a);
-    else lse_simt_kernel<false><<<grid, kSThreads, smem, st>>>(a);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? ESTP_OK : cuda_fail(e, "lse launch");
+    return launch_lse_f32(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen, lse, st, 0);
 }
 
 estp_status launch_importance(estp_ctx* ctx, const void* Q, const void* K, estp_dtype dtype,
                               const float* lse, int Hq, int Hkv, int d, float scale,
-                              const ImpHeads& hs, const int32_t* cu, int B, int64_t sumT,
+                              const ImpHeads& heads, const int32_t* cu, int B, int64_t sumT,
                               int max_seqlen, bool accumulate, uint32_t flags, float* acc,
                               cudaStream_t st) {
     const bool tc = tc_supported(dtype, d);
-    const int tile = tc ? tc_tile() : kSTile;
-    const int qc = tc ? tc_qc(B, sumT, hs.n_groups, ctx->num_sms) : kSQc;
+    const F32Split split = f32_split(B, sumT, heads, ctx->num_sms);
+    const bool apart = !tc && split.per_head;
+    const ImpHeads hs = apart ? heads_apart(heads, Hq / Hkv) : heads;
+    const int tile = tc ? tc_tile() : split.rows;
+    const int qc = tc ? tc_qc(B, sumT, hs.n_groups, ctx->num_sms) : split.qc;
     const int nt_max = (max_seqlen + tile - 1) / tile;
     const int c_max = nt_max > 0 ? chunks_of(nt_max, 0, qc) : 0;
     // workspace: [own lse][plan base][info][partials]
@@ -405,33 +462,15 @@ estp_status launch_importance(estp_ctx* ctx, const void* Q, const void* K, estp_
     estp_status s = ws_reserve(ctx, off_part + part_bytes);
     if (s != ESTP_OK) return s;
     char* ws = static_cast<char*>(ctx->ws);
-    // The LSE launch keeps its own plan at the start of the workspace, so an internal
-    // LSE goes first and sits below the importance plan.
+    // The LSE launch keeps its own plan in the workspace, which the importance plan then
+    // overwrites; its result sits below both.  It only needs rows of the selected heads.
     float* lse_use = const_cast<float*>(lse);
     if (!lse) {
         lse_use = reinterpret_cast<float*>(ws);
-        // LSE kernels only need rows of the selected heads.
-        if (tc) s = launch_lse_tc(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen,
-                                  lse_use, st, off_base);
-        else {
-            SimtArgs a{};
-            a.Q = Q; a.K = K; a.cu = cu; a.B = B; a.Hq = Hq; a.Hkv = Hkv; a.d = d; a.sumT = sumT;
-            a.base = reinterpret_cast<int32_t*>(ws + off_base);
-            a.info = reinterpret_cast<PlanInfo*>(ws + off_info);
-            a.scale_log2 = scale * kLog2e;
-            a.hs = hs;
-            a.lse_out = lse_use;
-            attn_plan_kernel<<<1, 1024, 0, st>>>(cu, B, sumT, max_seqlen, kSTile, 1, hs.n_heads, 1,
-                                                 reinterpret_cast<int32_t*>(ws + off_base),
-                                                 reinterpret_cast<PlanInfo*>(ws + off_info),
-                                                 ctx->status);
-            const size_t smem = simt_smem(d, false);
-            const void* kfn = dtype == ESTP_BF16 ? (const void*)lse_simt_kernel<true> : (const void*)lse_simt_kernel<false>;
-            cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            const int grid = persistent_grid(ctx, kfn, kSThreads, smem);
-            if (dtype == ESTP_BF16) lse_simt_kernel<true><<<grid, kSThreads, smem, st>>>(a);
-            else lse_simt_kernel<false><<<grid, kSThreads, smem, st>>>(a);
-        }
+        s = tc ? launch_lse_tc(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen, lse_use,
+                               st, off_base)
+               : launch_lse_f32(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen, lse_use,
+                                st, off_base);
         if (s != ESTP_OK) return s;
     }
     int32_t* base = reinterpret_cast<int32_t*>(ws + off_base);
@@ -444,17 +483,15 @@ estp_status launch_importance(estp_ctx* ctx, const void* Q, const void* K, estp_
                           (flags & ESTP_IMP_EXCLUDE_SELF) != 0, base, info, part, c_max, qc, st);
         if (s != ESTP_OK) return s;
     } else {
-        SimtArgs a{};
-        a.Q = Q; a.K = K; a.lse = lse_use; a.cu = cu; a.base = base; a.info = info; a.B = B;
+        F32Args a{};
+        a.Q = static_cast<const float*>(Q); a.K = static_cast<const float*>(K);
+        a.lse = lse_use; a.cu = cu; a.base = base; a.info = info; a.B = B;
         a.Hq = Hq; a.Hkv = Hkv; a.d = d; a.sumT = sumT; a.scale_log2 = scale * kLog2e;
-        a.hs = hs; a.exclude_self = (flags & ESTP_IMP_EXCLUDE_SELF) != 0; a.part = part;
-        a.c_max = c_max; a.status = ctx->status;
-        const size_t smem = simt_smem(d, true);
-        const void* kfn = dtype == ESTP_BF16 ? (const void*)imp_simt_kernel<true> : (const void*)imp_simt_kernel<false>;
-        cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        const int grid = persistent_grid(ctx, kfn, kSThreads, smem);
-        if (dtype == ESTP_BF16) imp_simt_kernel<true><<<grid, kSThreads, smem, st>>>(a);
-        else imp_simt_kernel<false><<<grid, kSThreads, smem, st>>>(a);
+        a.hs = hs; a.exclude_self = (flags & ESTP_IMP_EXCLUDE_SELF) ? 1 : 0; a.qc = qc;
+        a.part = part; a.c_max = c_max; a.status = ctx->status;
+        const cudaError_t e = tile == 128 ? launch_f32(ctx, imp_f32_kernel<8>, a, st)
+                                          : launch_f32(ctx, imp_f32_kernel<4>, a, st);
+        if (e != cudaSuccess) return cuda_fail(e, "importance launch");
     }
     {  // a programmatic dependent of the column-sum kernel: it waits on it on the device
         cudaLaunchAttribute attr[1];

@@ -7,7 +7,8 @@
 // one is multiplied.  Each thread holds TM x TN sums as packed pairs (fma.rn.f32x2: two FMAs
 // per issue slot, which leaves the other slots to the shared loads).  The sums of every 64
 // values of k are formed on their own and then added to the running ones, so that a sum over
-// k has chains of 64 and k / 64 additions and not one of k.
+// k has chains of 64 and k / 64 additions and not one of k.  (kChains = false leaves that out, for short sums of at
+// most 128 terms: half the registers.)
 #pragma once
 #include "estp_internal.cuh"
 
@@ -23,7 +24,7 @@ struct GemmSide {
     int vec;
 };
 
-template <int TM, int TN, int BK, bool kAlongA, bool kAlongB>
+template <int TM, int TN, int BK, bool kAlongA, bool kAlongB, bool kChains = true>
 struct SgemmTile {
     static constexpr int kThreads = 256;
     static constexpr int BM = 16 * TM, BN = 16 * TN;
@@ -158,17 +159,19 @@ struct SgemmTile {
         load(k0);
         put(0);
         __syncthreads();
-        float2 p[TM][TN / 2];
+        float2 p[kChains ? TM : 1][TN / 2];
         int buf = 0, slices = 0;
         float part_a = 0.f;
         for (int64_t k = k0; k < k1; k += BK) {
             const bool more = k + BK < k1;
             if (more) load(k + BK);
             if (slices == 0) {
+                if constexpr (kChains) {
 #pragma unroll
-                for (int i = 0; i < TM; ++i)
+                    for (int i = 0; i < TM; ++i)
 #pragma unroll
-                    for (int j = 0; j < TN / 2; ++j) p[i][j] = make_float2(0.f, 0.f);
+                        for (int j = 0; j < TN / 2; ++j) p[i][j] = make_float2(0.f, 0.f);
+                }
                 part_a = 0.f;
             }
             const float* as = sm + buf * kSlice;
@@ -181,16 +184,20 @@ struct SgemmTile {
 #pragma unroll
                 for (int i = 0; i < TM; ++i)
 #pragma unroll
-                    for (int j = 0; j < TN / 2; ++j)
-                        p[i][j] = __ffma2_rn(make_float2(av[i], av[i]), make_float2(bv[2 * j], bv[2 * j + 1]), p[i][j]);
+                    for (int j = 0; j < TN / 2; ++j) {
+                        float2& sum = kChains ? p[kChains ? i : 0][j] : c[i][j];
+                        sum = __ffma2_rn(make_float2(av[i], av[i]), make_float2(bv[2 * j], bv[2 * j + 1]), sum);
+                    }
                 if (kSumA && threadIdx.x < BM) part_a += as[kk * SA + threadIdx.x];
             }
             if (++slices == 64 / BK || !more) {
                 slices = 0;
+                if constexpr (kChains) {
 #pragma unroll
-                for (int i = 0; i < TM; ++i)
+                    for (int i = 0; i < TM; ++i)
 #pragma unroll
-                    for (int j = 0; j < TN / 2; ++j) c[i][j] = __fadd2_rn(c[i][j], p[i][j]);
+                        for (int j = 0; j < TN / 2; ++j) c[i][j] = __fadd2_rn(c[i][j], p[i][j]);
+                }
                 if (kSumA) *sum_a += part_a;
             }
             if (more) put(buf ^ 1);

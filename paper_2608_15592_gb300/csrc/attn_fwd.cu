@@ -652,34 +652,32 @@ estp_status launch_attn_forward(estp_ctx* ctx, const void* Q, const void* K, con
     const int64_t slots_bound = (int64_t)Hq * tiles_bound * (max_nt + 1) / 2 + Hq;
     const size_t off_part = 0;
     const size_t off_lse = off_part + align_up(sizeof(float) * (size_t)slots_bound * kT, 256);
-    const size_t off_plan = off_lse + (lse_in ? 0 : align_up(sizeof(float) * (size_t)Hq * sumT, 256));
-    const size_t off_base2 = off_plan + align_up(sizeof(int32_t) * (size_t)(B + 1), 256);
-    const size_t off_info = off_base2 + align_up(sizeof(int32_t) * (size_t)(B + 1), 256);
-    const size_t off_info2 = off_info + 256;
-    const size_t off_lse_plan = off_info2 + 256;
-    // the row-normaliser kernel's own plan comes after ours: reserve for it too
-    estp_status s = ws_reserve(ctx, off_lse_plan + align_up(sizeof(int32_t) * (size_t)(B + 1), 256) +
-                                        sizeof(PlanInfo) + 256);
+    const size_t off_items = off_lse + (lse_in ? 0 : align_up(sizeof(float) * (size_t)Hq * sumT, 256));
+    const size_t off_slots = off_items + plan_bytes(B);
+    const size_t off_lse_plan = off_slots + plan_bytes(B);
+    estp_status s = ws_reserve(ctx, off_lse_plan + plan_bytes(B));
     if (s != ESTP_OK) return s;
     char* ws = static_cast<char*>(ctx->ws);
     float* part = reinterpret_cast<float*>(ws + off_part);
-    int32_t* base = reinterpret_cast<int32_t*>(ws + off_plan);
-    int32_t* base2 = reinterpret_cast<int32_t*>(ws + off_base2);
-    PlanInfo* info = reinterpret_cast<PlanInfo*>(ws + off_info);
-    PlanInfo* info2 = reinterpret_cast<PlanInfo*>(ws + off_info2);
+    int32_t* base = plan_base(ws + off_items);
+    int32_t* base2 = plan_base(ws + off_slots);
+    PlanInfo* info = plan_info(ws + off_items, B);
+    PlanInfo* info2 = plan_info(ws + off_slots, B);
+    // plans: items (prompt, query tile, head), and the partial slots (tile pairs x heads)
+    const PlanReq items{kT, 1, Hq, 1, base, info}, slots{kT, 1, Hq, 2, base2, info2};
     const float* lse = lse_in;
-    if (!lse_in) {  // pass 1: the row normalisers of every head
+    if (lse_in) {
+        launch_plans(ctx, cu, B, sumT, max_seqlen, st, items, slots);
+    } else {  // pass 1: the row normalisers of every head, with their plan in the same launch
         float* l = reinterpret_cast<float*>(ws + off_lse);
         ImpHeads all;
         if ((s = build_heads(nullptr, Hq, Hq, Hkv, &all)) != ESTP_OK) return s;
-        if ((s = launch_lse_tc(ctx, Q, K, Hq, Hkv, kD, scale, all, cu, B, sumT, max_seqlen, l, st,
-                               off_lse_plan)) != ESTP_OK)
+        const PlanReq lp = lse_plan_tc(all, plan_base(ws + off_lse_plan), plan_info(ws + off_lse_plan, B));
+        launch_plans(ctx, cu, B, sumT, max_seqlen, st, items, slots, lp);
+        if ((s = launch_lse_tc(ctx, Q, K, Hq, Hkv, kD, scale, all, cu, B, sumT, l, lp, st)) != ESTP_OK)
             return s;
         lse = l;
     }
-    // plans: items (prompt, query tile, head), and the partial slots (tile pairs x heads)
-    attn_plan2_kernel<<<2, 1024, 0, st>>>(cu, B, sumT, max_seqlen, kT, 1, Hq, 1, base, info, 2, base2,
-                                          info2, ctx->status);
     // the forward and the reduce are programmatic dependents of the launch before them:
     // each starts its prologue early and waits on the device for its inputs
     cudaLaunchAttribute pdl[1];

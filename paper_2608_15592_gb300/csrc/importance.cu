@@ -74,24 +74,13 @@ static __device__ void plan_body(const int32_t* cu, int B, int64_t sumT, int max
 }
 
 __global__ void __launch_bounds__(1024) attn_plan_kernel(const int32_t* cu, int B, int64_t sumT,
-                                                         int max_seqlen, int tile, int qc,
-                                                         int mult, int kind, int32_t* base,
-                                                         PlanInfo* info, int* status) {
+                                                         int max_seqlen, const PlanSet plans,
+                                                         int* status) {
     // the tensor-core kernel that consumes the plan may launch now and run its prologue;
     // it waits for this grid before its first read of the plan
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    plan_body(cu, B, sumT, max_seqlen, tile, qc, mult, kind, base, info, status);
-}
-
-__global__ void __launch_bounds__(1024) attn_plan2_kernel(const int32_t* cu, int B, int64_t sumT,
-                                                          int max_seqlen, int tile, int qc,
-                                                          int mult, int kind0, int32_t* base0,
-                                                          PlanInfo* info0, int kind1,
-                                                          int32_t* base1, PlanInfo* info1,
-                                                          int* status) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (blockIdx.x == 0) plan_body(cu, B, sumT, max_seqlen, tile, qc, mult, kind0, base0, info0, status);
-    else plan_body(cu, B, sumT, max_seqlen, tile, qc, mult, kind1, base1, info1, status);
+    const PlanReq p = plans.plan[blockIdx.x];
+    plan_body(cu, B, sumT, max_seqlen, p.tile, p.qc, p.mult, p.kind, p.base, p.info, status);
 }
 
 namespace {
@@ -406,25 +395,32 @@ cudaError_t launch_f32(estp_ctx* ctx, Kernel kernel, const F32Args& a, cudaStrea
     return cudaGetLastError();
 }
 
-// Row normalisers of the selected heads (fp32), with the plan at byte ws_off of the workspace.
+PlanReq lse_plan_f32(const ImpHeads& hs, int B, int64_t sumT, int num_sms, int32_t* base,
+                     PlanInfo* info) {
+    return {f32_rows(B, sumT, hs.n_heads, num_sms), 1, hs.n_heads, 1, base, info};
+}
+
+// Row normalisers of the selected heads (fp32).
 estp_status launch_lse_f32(estp_ctx* ctx, const void* Q, const void* K, int Hq, int Hkv, int d,
                            float scale, const ImpHeads& hs, const int32_t* cu, int B, int64_t sumT,
-                           int max_seqlen, float* lse, cudaStream_t st, size_t ws_off) {
-    char* ws = static_cast<char*>(ctx->ws) + ws_off;
+                           float* lse, const PlanReq& plan, cudaStream_t st) {
     F32Args a{};
     a.Q = static_cast<const float*>(Q); a.K = static_cast<const float*>(K);
     a.cu = cu; a.B = B; a.Hq = Hq; a.Hkv = Hkv; a.d = d; a.sumT = sumT;
-    a.info = reinterpret_cast<PlanInfo*>(ws + align_up(sizeof(int32_t) * (size_t)(B + 1), 256));
-    a.base = reinterpret_cast<int32_t*>(ws);
+    a.info = plan.info;
+    a.base = plan.base;
     a.scale_log2 = scale * kLog2e;
     a.hs = hs;
     a.lse_out = lse;
-    const int rows = f32_rows(B, sumT, hs.n_heads, ctx->num_sms);
-    attn_plan_kernel<<<1, 1024, 0, st>>>(cu, B, sumT, max_seqlen, rows, 1, hs.n_heads, 1,
-                                         reinterpret_cast<int32_t*>(ws), a.info, ctx->status);
-    const cudaError_t e = rows == 128 ? launch_f32(ctx, lse_f32_kernel<8>, a, st)
-                                      : launch_f32(ctx, lse_f32_kernel<4>, a, st);
+    const cudaError_t e = plan.tile == 128 ? launch_f32(ctx, lse_f32_kernel<8>, a, st)
+                                           : launch_f32(ctx, lse_f32_kernel<4>, a, st);
     return e == cudaSuccess ? ESTP_OK : cuda_fail(e, "lse launch");
+}
+
+PlanReq lse_plan(bool tc, estp_ctx* ctx, const ImpHeads& hs, int B, int64_t sumT, char* ws) {
+    int32_t* base = plan_base(ws);
+    PlanInfo* info = plan_info(ws, B);
+    return tc ? lse_plan_tc(hs, base, info) : lse_plan_f32(hs, B, sumT, ctx->num_sms, base, info);
 }
 
 }  // namespace
@@ -432,12 +428,13 @@ estp_status launch_lse_f32(estp_ctx* ctx, const void* Q, const void* K, int Hq, 
 estp_status launch_lse(estp_ctx* ctx, const void* Q, const void* K, estp_dtype dtype, int Hq,
                        int Hkv, int d, float scale, const ImpHeads& hs, const int32_t* cu,
                        int B, int64_t sumT, int max_seqlen, float* lse, cudaStream_t st) {
-    if (tc_supported(dtype, d))
-        return launch_lse_tc(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen, lse, st);
-    const size_t off_info = align_up(sizeof(int32_t) * (size_t)(B + 1), 256);
-    estp_status s = ws_reserve(ctx, off_info + sizeof(PlanInfo));
+    estp_status s = ws_reserve(ctx, plan_bytes(B));
     if (s != ESTP_OK) return s;
-    return launch_lse_f32(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen, lse, st, 0);
+    const bool tc = tc_supported(dtype, d);
+    const PlanReq plan = lse_plan(tc, ctx, hs, B, sumT, static_cast<char*>(ctx->ws));
+    launch_plans(ctx, cu, B, sumT, max_seqlen, st, plan);
+    return tc ? launch_lse_tc(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, lse, plan, st)
+              : launch_lse_f32(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, lse, plan, st);
 }
 
 estp_status launch_importance(estp_ctx* ctx, const void* Q, const void* K, estp_dtype dtype,
@@ -453,31 +450,30 @@ estp_status launch_importance(estp_ctx* ctx, const void* Q, const void* K, estp_
     const int qc = tc ? tc_qc(B, sumT, hs.n_groups, ctx->num_sms) : split.qc;
     const int nt_max = (max_seqlen + tile - 1) / tile;
     const int c_max = nt_max > 0 ? chunks_of(nt_max, 0, qc) : 0;
-    // workspace: [own lse][plan base][info][partials]
+    // workspace: [own lse][plan of the lse][plan][partials]
     const size_t lse_bytes = lse ? 0 : align_up(sizeof(float) * (size_t)Hq * (size_t)sumT, 256);
-    const size_t off_base = lse_bytes;
-    const size_t off_info = off_base + align_up(sizeof(int32_t) * (size_t)(B + 1), 256);
-    const size_t off_part = off_info + 256;
+    const size_t off_lse_plan = lse_bytes;
+    const size_t off_plan = off_lse_plan + plan_bytes(B);
+    const size_t off_part = off_plan + plan_bytes(B);
     const size_t part_bytes = sizeof(float) * (size_t)c_max * (size_t)hs.n_groups * (size_t)sumT;
     estp_status s = ws_reserve(ctx, off_part + part_bytes);
     if (s != ESTP_OK) return s;
     char* ws = static_cast<char*>(ctx->ws);
-    // The LSE launch keeps its own plan in the workspace, which the importance plan then
-    // overwrites; its result sits below both.  It only needs rows of the selected heads.
+    int32_t* base = plan_base(ws + off_plan);
+    PlanInfo* info = plan_info(ws + off_plan, B);
+    float* part = reinterpret_cast<float*>(ws + off_part);
+    const PlanReq plan{tile, qc, hs.n_groups, 0, base, info};
     float* lse_use = const_cast<float*>(lse);
-    if (!lse) {
+    if (lse) {
+        launch_plans(ctx, cu, B, sumT, max_seqlen, st, plan);
+    } else {  // the rows of the selected heads first; both plans in one launch
         lse_use = reinterpret_cast<float*>(ws);
-        s = tc ? launch_lse_tc(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen, lse_use,
-                               st, off_base)
-               : launch_lse_f32(ctx, Q, K, Hq, Hkv, d, scale, hs, cu, B, sumT, max_seqlen, lse_use,
-                                st, off_base);
+        const PlanReq lp = lse_plan(tc, ctx, heads, B, sumT, ws + off_lse_plan);
+        launch_plans(ctx, cu, B, sumT, max_seqlen, st, lp, plan);
+        s = tc ? launch_lse_tc(ctx, Q, K, Hq, Hkv, d, scale, heads, cu, B, sumT, lse_use, lp, st)
+               : launch_lse_f32(ctx, Q, K, Hq, Hkv, d, scale, heads, cu, B, sumT, lse_use, lp, st);
         if (s != ESTP_OK) return s;
     }
-    int32_t* base = reinterpret_cast<int32_t*>(ws + off_base);
-    PlanInfo* info = reinterpret_cast<PlanInfo*>(ws + off_info);
-    float* part = reinterpret_cast<float*>(ws + off_part);
-    attn_plan_kernel<<<1, 1024, 0, st>>>(cu, B, sumT, max_seqlen, tile, qc, hs.n_groups, 0, base,
-                                         info, ctx->status);
     if (tc) {
         s = launch_imp_tc(ctx, Q, K, lse_use, Hq, Hkv, d, scale, hs, cu, B, sumT,
                           (flags & ESTP_IMP_EXCLUDE_SELF) != 0, base, info, part, c_max, qc, st);

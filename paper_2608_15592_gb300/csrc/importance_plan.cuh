@@ -34,21 +34,36 @@ __host__ __device__ __forceinline__ int64_t plan_count(int64_t nt, int qc, int k
     return kind == 0 ? items_f(nt, qc) : kind == 1 ? nt : nt * (nt + 1) / 2;
 }
 
-// Prefix of per-prompt counts (base[B+1]) and validation.  One CTA of 1024.
-// Each prompt counts mult * plan_count(nt, qc, kind).
-__global__ void __launch_bounds__(1024) attn_plan_kernel(const int32_t* cu, int B, int64_t sumT,
-                                                         int max_seqlen, int tile, int qc,
-                                                         int mult, int kind, int32_t* base,
-                                                         PlanInfo* info, int* status);
+// One plan: each prompt counts mult * plan_count(ceil(length / tile), qc, kind) items.
+struct PlanReq {
+    int tile, qc, mult, kind;
+    int32_t* base;   // [B + 1] prefix of the counts
+    PlanInfo* info;
+};
+constexpr int kMaxPlans = 3;
+struct PlanSet {
+    PlanReq plan[kMaxPlans];
+};
 
-// Two plans of the same prompts in one launch of 2 blocks: block 0 writes (kind0, base0,
-// info0), block 1 (kind1, base1, info1).
-__global__ void __launch_bounds__(1024) attn_plan2_kernel(const int32_t* cu, int B, int64_t sumT,
-                                                          int max_seqlen, int tile, int qc,
-                                                          int mult, int kind0, int32_t* base0,
-                                                          PlanInfo* info0, int kind1,
-                                                          int32_t* base1, PlanInfo* info1,
-                                                          int* status);
+// The plans a call's kernels need and the validation of cu_seqlens, in one launch of a block
+// of 1024 threads each.
+__global__ void __launch_bounds__(1024) attn_plan_kernel(const int32_t* cu, int B, int64_t sumT,
+                                                         int max_seqlen, const PlanSet plans,
+                                                         int* status);
+template <class... Plans>
+void launch_plans(estp_ctx* ctx, const int32_t* cu, int B, int64_t sumT, int max_seqlen,
+                  cudaStream_t st, const Plans&... plans) {
+    static_assert(sizeof...(plans) <= kMaxPlans, "plans of one call");
+    attn_plan_kernel<<<sizeof...(plans), 1024, 0, st>>>(cu, B, sumT, max_seqlen, PlanSet{{plans...}},
+                                                        ctx->status);
+}
+
+// Workspace bytes of a plan, and its two parts.
+inline size_t plan_bytes(int B) { return align_up(sizeof(int32_t) * (size_t)(B + 1), 256) + 256; }
+inline int32_t* plan_base(char* ws) { return reinterpret_cast<int32_t*>(ws); }
+inline PlanInfo* plan_info(char* ws, int B) {
+    return reinterpret_cast<PlanInfo*>(ws + plan_bytes(B) - 256);
+}
 
 struct ImpItem {
     int b, g, kt, qt0, qt1;

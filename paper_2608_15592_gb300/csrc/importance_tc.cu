@@ -736,8 +736,9 @@ estp_status launch_tc(estp_ctx* ctx, const CUtensorMap& fixm, const CUtensorMap&
     const int smem = Cfg<D>::kSmemBytes;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_fail(e, "tc kernel smem attribute");
-    // a programmatic dependent of the plan kernel: the launch and the prologue (barriers,
-    // TMEM, tensor-map prefetch) overlap the plan, which the kernel waits for on the device
+    // a programmatic dependent of the plan kernel or of the row normalisers: the launch and the
+    // prologue (barriers, TMEM, tensor-map prefetch) overlap it, and the kernel waits for it on
+    // the device (no CTA shares an SM with one of the row normalisers: shared memory)
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -767,34 +768,36 @@ int tc_qc(int B, int64_t sumT, int n_groups, int num_sms) {
     return kQcChoices[3];
 }
 
+// LSE items: (prompt, query tile, pair of heads of one KV group) when every group holds an
+// even number of the selected heads, else (prompt, pair of query tiles, head)
+static bool lse_head_pairs(const ImpHeads& hs) {
+    for (int g = 0; g < hs.n_groups; ++g)
+        if ((hs.begin[g + 1] - hs.begin[g]) & 1) return false;
+    return true;
+}
+
+PlanReq lse_plan_tc(const ImpHeads& hs, int32_t* base, PlanInfo* info) {
+    return lse_head_pairs(hs) ? PlanReq{kTile, 1, hs.n_heads / 2, 1, base, info}
+                              : PlanReq{kPair, 1, hs.n_heads, 1, base, info};
+}
+
 estp_status launch_lse_tc(estp_ctx* ctx, const void* Q, const void* K, int Hq, int Hkv, int d,
                           float scale, const ImpHeads& hs, const int32_t* cu, int B, int64_t sumT,
-                          int max_seqlen, float* lse, cudaStream_t st, size_t ws_off) {
-    const size_t off_info = ws_off + align_up(sizeof(int32_t) * (size_t)(B + 1), 256);
-    estp_status s = ws_reserve(ctx, off_info + sizeof(PlanInfo));
-    if (s != ESTP_OK) return s;
-    char* ws = static_cast<char*>(ctx->ws);
+                          float* lse, const PlanReq& plan, cudaStream_t st) {
     TcArgs a{};
     a.cu = cu; a.B = B; a.Hq = Hq; a.Hkv = Hkv; a.sumT = sumT;
-    a.base = reinterpret_cast<int32_t*>(ws + ws_off);
-    a.info = reinterpret_cast<PlanInfo*>(ws + off_info);
+    a.base = plan.base;
+    a.info = plan.info;
     a.scale_log2 = scale * kLog2e;
     a.lse_out = lse;
     a.status = ctx->status;
     a.wait_cycles = ctx->wait_cycles;
     a.hs = hs;
+    a.head_pairs = lse_head_pairs(hs) ? 1 : 0;
     CUtensorMap mq, mk;
+    estp_status s;
     if ((s = make_map(&mq, Q, Hq, d, sumT)) != ESTP_OK) return s;
     if ((s = make_map(&mk, K, Hkv, d, sumT)) != ESTP_OK) return s;
-    // LSE items: (prompt, query tile, pair of heads of one KV group) when every group holds
-    // an even number of the selected heads, else (prompt, pair of query tiles, head)
-    a.head_pairs = 1;
-    for (int g = 0; g < hs.n_groups; ++g)
-        if ((hs.begin[g + 1] - hs.begin[g]) & 1) a.head_pairs = 0;
-    attn_plan_kernel<<<1, 1024, 0, st>>>(cu, B, sumT, max_seqlen, a.head_pairs ? kTile : kPair, 1,
-                                         a.head_pairs ? hs.n_heads / 2 : hs.n_heads, 1,
-                                         const_cast<int32_t*>(a.base), const_cast<PlanInfo*>(a.info),
-                                         ctx->status);
     // (the lse map argument is unused in this mode)
     return d == 64 ? launch_tc<64, kModeLse>(ctx, mq, mk, mq, a, st)
                    : launch_tc<128, kModeLse>(ctx, mq, mk, mq, a, st);

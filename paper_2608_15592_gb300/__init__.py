@@ -137,9 +137,13 @@ def _ptr(t) -> int | None:
 
 
 def _stream(stream) -> int | None:
+    if stream is not None:
+        return stream.cuda_stream or None
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream or None
+    if not torch.cuda.is_initialized():
+        torch.cuda.init()
+    # the handle alone: building the Stream object that wraps it costs 2.9 us a call, this 0.5
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
 
 
 @dataclass
@@ -167,10 +171,17 @@ class Context:
 
     def __init__(self, device: int = 0, library=None):
         self.device = device
+        self._dev = None  # the torch.device, built at its first use
         self._lib = lib if library is None else library
         h = ctypes.c_void_p()
         self._check(self._lib.estp_create(ctypes.byref(h), device))
         self._h = h
+
+    def _torch_device(self):
+        if self._dev is None:
+            import torch
+            self._dev = torch.device("cuda", self.device)
+        return self._dev
 
     def _check(self, status: int):
         if status != ESTP_OK:
@@ -289,7 +300,7 @@ class Context:
         import torch
         if out is None:
             out = torch.empty(sumT, dtype=torch.float32,
-                              device=device if device is not None else f"cuda:{self.device}")
+                              device=device if device is not None else self._torch_device())
         self._check(self._lib.estp_attn_importance_finalize(self._h, n_layers, _ptr(out), _stream(stream)))
         return out
 
@@ -316,14 +327,14 @@ class Context:
         gW = torch.empty(K, D, dtype=torch.float32, device=dev) if grads else None
         gb = torch.empty(K, dtype=torch.float32, device=dev) if grads else None
         gp = torch.empty(B, D, dtype=torch.float32, device=dev) if grads else None
-        hp = ctypes.pointer(_Head(_ptr(head.W), _ptr(head.bias), _ptr(head.centers), K))
+        hp = ctypes.byref(_Head(_ptr(head.W), _ptr(head.bias), _ptr(head.centers), K))
         self._check(self._lib.estp_head_loss(self._h, _ptr(pooled), B, D, hp, _ptr(targets), lambda3,
                                   _ptr(loss), _ptr(gW), _ptr(gb), _ptr(gp), _stream(stream)))
         return (loss, gW, gb, gp) if grads else loss
 
     @staticmethod
     def _mlp(head: "MlpHead"):
-        return ctypes.pointer(_MlpHead(_ptr(head.W1), _ptr(head.b1), _ptr(head.W2), _ptr(head.b2),
+        return ctypes.byref(_MlpHead(_ptr(head.W1), _ptr(head.b1), _ptr(head.W2), _ptr(head.b2),
                                        _ptr(head.centers), head.W1.shape[0], head.W2.shape[0]))
 
     def mlp_head_predict(self, pooled, head: "MlpHead", probs: bool = False, stream=None):
@@ -350,7 +361,7 @@ class Context:
         out = {k: torch.empty(v, dtype=torch.float32, device=dev) if k in want else None
                for k, v in shapes.items()}
         loss = torch.empty(1, dtype=torch.float32, device=dev)
-        gp = ctypes.pointer(_MlpGrads(*[_ptr(out[k]) for k in ("W1", "b1", "W2", "b2", "pooled")]))
+        gp = ctypes.byref(_MlpGrads(*[_ptr(out[k]) for k in ("W1", "b1", "W2", "b2", "pooled")]))
         self._check(self._lib.estp_mlp_head_loss(self._h, _ptr(pooled), B, D, self._mlp(head), _ptr(targets),
                                       lambda3, _ptr(loss), gp if want else None, _stream(stream)))
         if not grads:
@@ -372,7 +383,7 @@ class Context:
         hp = None
         if head is not None:
             pred = torch.empty(B, dtype=torch.float32, device=dev) if pred is None else pred
-            hp = ctypes.pointer(_Head(_ptr(head.W), _ptr(head.bias), _ptr(head.centers),
+            hp = ctypes.byref(_Head(_ptr(head.W), _ptr(head.bias), _ptr(head.centers),
                                       head.W.shape[0]))
         mix = MixParams(lambda1, lambda2, alpha)
         self._check(self._lib.estp_pool(self._h, _ptr(hidden), _dtype(hidden), D, ldh, _ptr(entropy),

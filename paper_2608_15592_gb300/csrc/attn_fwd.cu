@@ -160,8 +160,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     attn_fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                     const __grid_constant__ CUtensorMap tm_v, const FwdArgs a) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~uintptr_t(1023));
+    // an offset, not a rounded address: the compiler then knows the pointer as shared memory
+    uint8_t* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);
     float* cs = reinterpret_cast<float*>(sm + kCsOff);
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kBarOff);
     uint64_t* q_full = bars;                         // [kQBufs]

@@ -79,18 +79,22 @@ __device__ __forceinline__ ImpItem decode_imp_item_at(int item, int b, const int
     it.t0 = cu[it.b];
     it.T = cu[it.b + 1] - cu[it.b];
     const int nt = (it.T + tile - 1) / tile;
-    const int64_t per_group = items_f(nt, qc);
-    const int64_t local = item - base[it.b];
+    // a plan holds fewer than 2^30 items, so 32 bits do (a 64-bit division costs ~100 instructions)
+    auto f = [qc](uint32_t n) {
+        const uint32_t a = n / (uint32_t)qc, r = n % (uint32_t)qc;
+        return (uint32_t)qc * (a * (a + 1) / 2) + r * (a + 1);
+    };
+    const uint32_t per_group = f((uint32_t)nt);
+    const uint32_t local = (uint32_t)(item - base[it.b]);
     it.g = (int)(local / per_group);
-    const int64_t rem = local - (int64_t)it.g * per_group;
-    const int64_t fnt = per_group;
+    const uint32_t rem = local - (uint32_t)it.g * per_group;
     int lo = 0, hi = nt - 1;  // largest kt with F(kt) <= rem
     while (lo < hi) {
         int mid = (lo + hi + 1) >> 1;
-        if (fnt - items_f(nt - mid, qc) <= rem) lo = mid; else hi = mid - 1;
+        if (per_group - f((uint32_t)(nt - mid)) <= rem) lo = mid; else hi = mid - 1;
     }
     it.kt = lo;
-    const int c = (int)(rem - (fnt - items_f(nt - lo, qc)));
+    const int c = (int)(rem - (per_group - f((uint32_t)(nt - lo))));
     it.qt0 = lo + c * qc;
     it.qt1 = min(nt, it.qt0 + qc);
     return it;

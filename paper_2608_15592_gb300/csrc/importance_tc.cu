@@ -57,7 +57,8 @@ constexpr int kEpiWarps = 16;          // 8 per fixed tile (LSE) or 4 per tile a
 // MMA issuers: warp 1 for fixed tile A, warp 18 for tile B, so that one issuer's barrier
 // waits and commits overlap the other's MMAs in the tensor pipe
 constexpr int kMmaWarpB = kEpiWarp0 + kEpiWarps;
-constexpr int kThreads = 32 * (kMmaWarpB + 1);
+constexpr int kNlWarp = kMmaWarpB + 1;  // column sums: prepares each step's row normalisers
+constexpr int threads_of(int mode) { return 32 * (mode == 1 ? kNlWarp + 1 : kNlWarp); }
 constexpr int kAccCols = 128;
 constexpr int kAccBufs = 2;            // accumulator pairs in TMEM (kAccBufs x 2 x 128 columns)
 constexpr int kSched = 4;              // depth of the item-index ring (producer -> consumers)
@@ -70,6 +71,19 @@ constexpr int kLseSlotBytes = 640;     // >= kLseBox * 4, multiple of 128
 
 enum Mode { kModeLse = 0, kModeImp = 1 };
 
+// --------------------------------------------------------------- item description
+// Decoded once, by the producer, and read by the other roles from the schedule ring.
+struct alignas(16) TcItem {
+    int64_t t0;
+    int valid, T;              // valid = 0: no more items
+    int fix_y, fix_row0;       // fixed tile A: head (LSE: query head, IMP: KV head), first row
+    int fix_y2, dq;            // fixed tile B: head, and its tile offset from A (1 or 0)
+    int n_steps;
+    // LSE: the query heads of tiles A and B and tile A's query tile (qt0);
+    // IMP: group slot, the pair's first key tile (kt), query-tile range, chunk slot
+    int h, h2, g, kt, qt0, qt1, chunk;
+};
+
 template <int D>
 struct Cfg {
     static constexpr int kAtoms = D / 64;
@@ -78,16 +92,16 @@ struct Cfg {
     // dynamic smem layout (offsets from a 1024-aligned base)
     static constexpr int kFixOff = 0;                               // [2 buffers][A, B]
     static constexpr int kRingOff = 4 * kTileBytes;
-    static constexpr int kNlOff = kRingOff + kStages * kTileBytes;  // [16 warps][128] f32
-    static constexpr int kMergeOff = kNlOff + kEpiWarps * 128 * 4;   // [2][A, B][4][32] float2
+    static constexpr int kNlOff = kRingOff + kStages * kTileBytes;  // [kAccBufs][128] f32
+    static constexpr int kMergeOff = kNlOff + kAccBufs * kTile * 4;   // [2][A, B][4][32] float2
     static constexpr int kBarOff = kMergeOff + 2 * 2 * 4 * 32 * 8;
     // fix_full/empty[2], ring_full/empty[kStages], acc_full/empty[A, B][kAccBufs],
     // drain[A, B], sched_full/empty[kSched], xfull/xempty[2][A, B][4], lse_full/empty[kLseSlots]
     static constexpr int kNumBars =
         2 + 2 + 2 * kStages + 4 * kAccBufs + 2 + 2 * kSched + 32 + 2 * kLseSlots;
-    // tmem addr, abort flag, then the sched ring's item indices and their prompts (int32)
-    static constexpr int kMiscOff = kBarOff + kNumBars * 8;
-    static constexpr int kLseOff = (kMiscOff + 16 + 8 * kSched + 127) / 128 * 128;  // lse ring
+    // tmem addr, abort flag, then the sched ring's items
+    static constexpr int kMiscOff = (kBarOff + kNumBars * 8 + 15) / 16 * 16;
+    static constexpr int kLseOff = (kMiscOff + 16 + (int)sizeof(TcItem) * kSched + 127) / 128 * 128;  // lse ring
     static constexpr int kSmemBytes = kLseOff + kLseSlots * kLseSlotBytes + 1024;  // + alignment slack
 };
 
@@ -113,29 +127,18 @@ struct TcArgs {
 // Instruction descriptor: M = N = 128.
 constexpr uint32_t kIdesc = idesc_bf16(kTile, kTile);
 
-// --------------------------------------------------------------- item description
-struct TcItem {
-    int b, T;
-    int64_t t0;
-    int fix_y, fix_row0;       // fixed tile A: head (LSE: query head, IMP: KV head), first row
-    int fix_y2, dq;            // fixed tile B: head, and its tile offset from A (1 or 0)
-    int n_steps;
-    // LSE: the query heads of tiles A and B and tile A's query tile (qt0);
-    // IMP: group slot, the pair's first key tile (kt), query-tile range, chunk slot
-    int h, h2, g, kt, qt0, qt1, chunk;
-};
-
-// Item `item`, which belongs to prompt b (looked up once by the producer).
+// Item `item`, which belongs to prompt b.
 template <int MODE>
 __device__ __forceinline__ TcItem make_item(const TcArgs& a, int item, int b) {
     TcItem t;
+    t.valid = 1;
     if (MODE == kModeLse) {
         t.g = 0; t.kt = 0; t.chunk = 0;
         if (a.head_pairs) {
             // Query tile qt0 of heads head_list[2u] (A) and head_list[2u + 1] (B), two heads of
             // one KV group: both need the key tiles 0 .. qt0, so no step leaves a tile idle.
             const LseItem li = decode_lse_item_at(item, b, a.base, a.cu, kTile, a.hs.n_heads >> 1);
-            t.b = li.b; t.T = li.T; t.t0 = li.t0;
+            t.T = li.T; t.t0 = li.t0;
             t.h = a.hs.head_list[2 * li.hslot];
             t.h2 = a.hs.head_list[2 * li.hslot + 1];
             t.qt0 = li.qt;
@@ -143,7 +146,7 @@ __device__ __forceinline__ TcItem make_item(const TcArgs& a, int item, int b) {
             t.n_steps = t.qt0 + 1;
         } else {
             const LseItem li = decode_lse_item_at(item, b, a.base, a.cu, kPair, a.hs.n_heads);
-            t.b = li.b; t.T = li.T; t.t0 = li.t0;
+            t.T = li.T; t.t0 = li.t0;
             t.h = t.h2 = a.hs.head_list[li.hslot];
             const int nt = (t.T + kTile - 1) / kTile;
             // Query tiles qt0 (A) and qt0 + 1 (B).  Pairs end at the prompt's last tile, so
@@ -159,7 +162,7 @@ __device__ __forceinline__ TcItem make_item(const TcArgs& a, int item, int b) {
         t.qt1 = t.qt0 + 1 + t.dq;
     } else {
         const ImpItem ii = decode_imp_item_at(item, b, a.base, a.cu, kPair, a.qc);
-        t.b = ii.b; t.T = ii.T; t.t0 = ii.t0;
+        t.T = ii.T; t.t0 = ii.t0;
         const int nt = (t.T + kTile - 1) / kTile;
         t.g = ii.g;
         t.kt = 2 * ii.kt;                  // key tiles kt (A) and kt + 1 (B, may be >= nt)
@@ -215,13 +218,13 @@ struct StepIter {
 };
 
 template <int D, int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(threads_of(MODE), 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tm_fix, const __grid_constant__ CUtensorMap tm_str,
                    const __grid_constant__ CUtensorMap tm_lse, const TcArgs a) {
     using C = Cfg<D>;
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~uintptr_t(1023));
+    // an offset, not a rounded address: the compiler then knows the pointer as shared memory
+    uint8_t* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);
     uint8_t* fix = sm + C::kFixOff;
     uint8_t* ring = sm + C::kRingOff;
     float* nl_all = reinterpret_cast<float*>(sm + C::kNlOff);
@@ -243,8 +246,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     float* lse_ring = reinterpret_cast<float*>(sm + C::kLseOff);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + C::kMiscOff);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + C::kMiscOff + 4);
-    volatile int* sched_item = reinterpret_cast<volatile int*>(sm + C::kMiscOff + 16);
-    volatile int* sched_b = sched_item + kSched;  // prompt of each published item
+    TcItem* sched_item = reinterpret_cast<TcItem*>(sm + C::kMiscOff + 16);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -253,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&fix_empty[i], 2);  // both issuers
         }
         for (int i = 0; i < 2 * kAccBufs; ++i) {
-            mbar_init(&acc_full[i], 1);
+            mbar_init(&acc_full[i], MODE == kModeImp ? 2 : 1);  // the issuer; the normaliser warp
             mbar_init(&acc_empty[i], MODE == kModeLse ? kEpiWarps / 2 : kEpiWarps / 4);  // its readers
         }
         for (int i = 0; i < C::kStages; ++i) {
@@ -264,7 +266,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_init(&drain[1], 1);
         for (int i = 0; i < kSched; ++i) {
             mbar_init(&sched_full[i], 1);
-            mbar_init(&sched_empty[i], 2 + kEpiWarps);  // MMA issuers + epilogue warps
+            // MMA issuers, epilogue warps and (column sums) the normaliser warp
+            mbar_init(&sched_empty[i], 2 + kEpiWarps + (MODE == kModeImp ? 1 : 0));
         }
         for (int i = 0; i < 16; ++i) {
             mbar_init(&xfull[i], 1);
@@ -272,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int i = 0; i < kLseSlots; ++i) {
             mbar_init(&lse_full[i], 1);
-            mbar_init(&lse_empty[i], kEpiWarps / 2);  // one arrival per warp that reads the step
+            mbar_init(&lse_empty[i], 1);  // the normaliser warp
         }
         *abort_flag = 0;
         mbar_fence_init();
@@ -295,20 +298,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     PlanInfo* info = const_cast<PlanInfo*>(a.info);
     const int total = info->total;
 
-    // Item k of this CTA and its prompt, published by the producer in slot k % kSched
-    // (item -1 = no more).
-    auto consume_item = [&](int k, bool warp_uniform, int& b) -> int {
+    // Item k of this CTA, published by the producer in slot k % kSched.
+    auto consume_item = [&](int k, bool warp_uniform) -> TcItem {
         const int slot = k % kSched;
         const uint32_t par = (uint32_t)((k / kSched) & 1);
         bool got;
         if (warp_uniform) got = warp_wait(&sched_full[slot], par, abort_flag, a.status, a.wait_cycles);
         else got = wait_bar(&sched_full[slot], par, abort_flag, a.status, a.wait_cycles);
-        if (!got) return -1;
-        const int item = sched_item[slot];
-        b = sched_b[slot];
+        TcItem t{};
+        if (!got) return t;
+        t = sched_item[slot];
         if (warp_uniform) __syncwarp();
         if (!warp_uniform || lane == 0) mbar_arrive(&sched_empty[slot]);
-        return item;
+        return t;
     };
 
     if (warp == 0) {
@@ -330,13 +332,11 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (it >= kSched &&
                     !wait_bar(&sched_empty[slot], (uint32_t)(((it / kSched) - 1) & 1), abort_flag, a.status, a.wait_cycles))
                     break;
-                // the item's prompt: one lookup here instead of one in every consumer role
-                const int b = item >= 0 ? upper_slot(a.base, a.B, item) : 0;
-                sched_item[slot] = item;
-                sched_b[slot] = b;
-                mbar_arrive(&sched_full[slot]);  // release: item and prompt visible to waiters
+                TcItem t{};
+                if (item >= 0) t = make_item<MODE>(a, item, upper_slot(a.base, a.B, item));
+                sched_item[slot] = t;
+                mbar_arrive(&sched_full[slot]);  // release: the item is visible to waiters
                 if (item < 0) break;
-                const TcItem t = make_item<MODE>(a, item, b);
                 const int fb = it & 1;
                 if (it >= 2 && !wait_bar(&fix_empty[fb], ((it >> 1) - 1) & 1, abort_flag, a.status, a.wait_cycles)) break;
                 mbar_expect_tx(&fix_full[fb], 2 * C::kTileBytes);
@@ -355,6 +355,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int stage = (int)(step % C::kStages);
                     const uint32_t u = step / C::kStages;
                     const int y = si.y, row0 = si.row0, head = si.head;
+                    // the next item is claimed before this one's last copies, which hide the
+                    // round trip of the atomic
+                    if (s == t.n_steps - 1) item = (int)gridDim.x + atomicAdd(&info->next, 1);
                     if (MODE == kModeImp) {  // the tile's lse values, from a 16-byte boundary
                         const int ls = (int)(step % kLseSlots);
                         const uint32_t lu = step / kLseSlots;
@@ -385,7 +388,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (!ok) break;
                 }
                 if (!ok) break;
-                item = (int)gridDim.x + atomicAdd(&info->next, 1);
             }
             // Every copy this thread issued has landed before the CTA can exit (on the
             // normal path the consumers already waited for all of them).
@@ -407,10 +409,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t step = 0;
             bool issued = false;
             for (int it = 0;; ++it) {
-                int b = 0;
-                const int item = consume_item(it, false, b);
-                if (item < 0) break;
-                const TcItem t = make_item<MODE>(a, item, b);
+                const TcItem t = consume_item(it, false);
+                if (!t.valid) break;
                 const int fb = it & 1;
                 if (!wait_bar(&fix_full[fb], (it >> 1) & 1, abort_flag, a.status, a.wait_cycles)) break;
                 const uint32_t fix_addr = smem_u32(fix + (fb * 2 + tau) * C::kTileBytes);
@@ -469,40 +469,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int col0 = MODE == kModeLse ? sub * 64 : 0;
         const int q = warp & 3;                    // TMEM lane quarter
         const int row = q * 32 + lane;             // accumulator row owned by this thread
-        float* nl = nl_all + e * 128;
         uint32_t step = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            int b = 0;
-            const int item = consume_item(it, true, b);
-            if (item < 0) break;
-            const TcItem t = make_item<MODE>(a, item, b);
+            const TcItem t = consume_item(it, true);
+            if (!t.valid) break;
             // column-sum mode: partial sums of this thread's four key rows 8 s + g8 (s = 0..3)
             // of the quarter, over its columns (16x256b layout, see below)
             float2 acc4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                               make_float2(0.f, 0.f)};
             float m = -1e30f, ssum = 0.f;          // LSE mode
-            StepIter<MODE> si(a, t);
+            int qt = t.qt0;                        // column sums: the step's query tile
             auto do_step = [&](int s) -> bool {
-                const int row0 = si.row0, head = si.head, qt = si.qt;
-                if (MODE == kModeImp) {  // -log2e * lse of the step's 128 query columns
-                    const int ls = (int)(step % kLseSlots);
-                    if (!warp_wait(&lse_full[ls], (step / kLseSlots) & 1, abort_flag, a.status, a.wait_cycles))
-                        return false;
-                    const int64_t x = (int64_t)head * a.sumT + t.t0 + row0;
-                    const float* lr = lse_ring + ls * (kLseSlotBytes / 4) + (int)(x & 3);
-                    float r[4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int i = row0 + 32 * k + lane;
-                        r[k] = i < t.T ? -lr[32 * k + lane] * kLog2e : -INFINITY;
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&lse_empty[ls]);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) nl[32 * k + lane] = r[k];
-                    __syncwarp();
-                }
                 const int ab = (int)(step % kAccBufs);
                 const int abar = tau * kAccBufs + ab;  // accumulator barrier
                 if (!warp_wait(&acc_full[abar], (step / kAccBufs) & 1, abort_flag, a.status, a.wait_cycles))
@@ -526,6 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((ab * 2 + tau) * kAccCols + col0);
                 const float2 sc = make_float2(a.scale_log2, a.scale_log2);
                 if constexpr (MODE == kModeImp) {
+                    const float* nl = nl_all + ab * kTile;  // -log2e * lse of the step's query columns
                     // 16x256b loads: thread (g8, c4) = (lane / 4, lane % 4) holds key rows
                     // q*32 + 16 lh + 8 jj + g8 and query columns 64 h + 8 k + 2 c4 + {0, 1}.
                     // Each query column's -lse log2e is then needed by 8 lanes only: 8
@@ -629,8 +608,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 return true;
                 }
             };
-            for (int s = 0; s < t.n_steps; ++s, ++step, si.next(a, t))
+            for (int s = 0; s < t.n_steps; ++s, ++step) {
                 if ((MODE == kModeLse || (int)(step & 1) == sub) && !(ok = do_step(s))) break;
+                if (MODE == kModeImp && ++qt == t.qt1) qt = t.qt0;
+            }
             if (!ok) break;
             // column-sum mode: the four lanes c4 of a g8 hold columns of the same four rows;
             // a butterfly over them gives each the rows' sums (the same bits in all four,
@@ -683,6 +664,46 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int h = tau ? t.h2 : t.h;
                     if (i >= 0 && i < t.T && in_bounds(h >= 0 && h < a.Hq && t.t0 + i < a.sumT, a.status))
                         a.lse_out[(int64_t)h * a.sumT + t.t0 + i] = (mm + lg2(ss)) * kLn2;
+                }
+            }
+        }
+    } else if (MODE == kModeImp && warp == kNlWarp) {
+        // ------------------------------------------------------ row normalisers
+        // -log2e * lse of every step's 128 query columns, -inf past the prompt, from the copied
+        // values to the buffer of the step's accumulators; the arrival on their barriers hands
+        // both over at once, and their release frees both.
+        uint32_t step = 0;
+        bool ok = true;
+        for (int it = 0; ok; ++it) {
+            const TcItem t = consume_item(it, true);
+            if (!t.valid) break;
+            StepIter<MODE> si(a, t);
+            for (int s = 0; s < t.n_steps; ++s, ++step, si.next(a, t)) {
+                const int ls = (int)(step % kLseSlots);
+                ok = warp_wait(&lse_full[ls], (step / kLseSlots) & 1, abort_flag, a.status, a.wait_cycles);
+                if (!ok) break;
+                const int64_t x = (int64_t)si.head * a.sumT + t.t0 + si.row0;
+                const float* lr = lse_ring + ls * (kLseSlotBytes / 4) + (int)(x & 3);
+                float r[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int i = si.row0 + 32 * k + lane;
+                    r[k] = i < t.T ? -lr[32 * k + lane] * kLog2e : -INFINITY;
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&lse_empty[ls]);
+                const int ab = (int)(step % kAccBufs);
+                const uint32_t use = step / kAccBufs;
+                if (use >= 1)
+                    ok = warp_wait(&acc_empty[ab], (use - 1) & 1, abort_flag, a.status, a.wait_cycles) &&
+                         warp_wait(&acc_empty[kAccBufs + ab], (use - 1) & 1, abort_flag, a.status, a.wait_cycles);
+                if (!ok) break;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) nl_all[ab * kTile + 32 * k + lane] = r[k];
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&acc_full[ab]);
+                    mbar_arrive(&acc_full[kAccBufs + ab]);
                 }
             }
         }
@@ -744,7 +765,7 @@ estp_status launch_tc(estp_ctx* ctx, const CUtensorMap& fixm, const CUtensorMap&
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctx->num_sms);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(threads_of(MODE));
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = st;
     cfg.attrs = attr;

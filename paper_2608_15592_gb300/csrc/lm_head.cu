@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     lm_head_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_b,
                    const __grid_constant__ CUtensorMap tm_bu, const LmArgs a) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                             ~uintptr_t(1023));
+    // an offset, not a rounded address: the compiler then knows the pointer as shared memory
+    uint8_t* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kBarOff);
     uint64_t* full = bars;                       // [kStages]
     uint64_t* empty = full + kStages;            // [kStages]

@@ -12,13 +12,17 @@
 //                D_B = B x S^T (warp 18), M = 128, N = 128, fp32 in TMEM, each
 //                double-buffered: 2 x 2 x 128 = all 512 TMEM columns
 //   warps 2-17   epilogue: tcgen05.ld, exp2 and row reductions; warp w reads TMEM lanes
-//                32*(w%4).. (its quarter).  LSE mode: 8 warps per fixed tile, two per
-//                quarter splitting the 128 columns, at every step.  Column-sum mode: a
-//                group of 4 warps per fixed tile and accumulator buffer reads all 128
-//                columns at every other step, so the two buffers' groups work a step
-//                apart and each step's lse values pass through 8 warps instead of 16
-//                (12 % faster there; in LSE mode the longer hold on the accumulator
-//                before it is released costs more than it gains)
+//                32*(w%4).. (its quarter).  8 warps per fixed tile, two per quarter, each with
+//                64 of the 128 columns at every step.  A warp loads its 64 columns whole and
+//                releases the accumulator before any arithmetic on them, so that the tensor
+//                pipe runs ahead of the exponentials (row normalisers 5.05 -> 4.79 ms on 256
+//                prompts against two loads of 32 with the release after the second)
+//   warp 19      column sums: -log2e * lse of each step's query tile, prepared once for the
+//                16 epilogue warps
+// What bounds it (one prompt of 32768, cycles a step of two tiles): the tensor pipe 1024, shared
+// memory ~1250 (operand reads and the TMA's writes), the epilogue's issue slots ~1390 to 1630;
+// a step takes 1680.
+//
 // Two issuers because the tensor core's instruction queue is shallow: a check of an
 // mbarrier costs an issuing thread ~150-180 cycles even when the phase has completed,
 // and with a single issuer the pipe idles through its two waits and commits per step;
@@ -39,6 +43,8 @@
 // ESTP_ERR_TIMEOUT in the status word, skips every further abortable wait, and drains:
 // the producer waits (full limit) for its last copies into each ring slot, fixed-tile
 // buffer and lse slot, the issuers for all their MMAs, before the TMEM is freed.
+#include <type_traits>
+
 #include "importance_tc.cuh"
 #include "tcgen05.cuh"
 
@@ -53,7 +59,7 @@ constexpr int kPair = 2 * kTile;       // rows of the fixed pair (the plan's til
 constexpr int kQcChoices[4] = {16, 8, 4, 2};
 constexpr int kItemsPerSm = 16;
 constexpr int kEpiWarp0 = 2;           // warps 2..17
-constexpr int kEpiWarps = 16;          // 8 per fixed tile (LSE) or 4 per tile and buffer (column sums)
+constexpr int kEpiWarps = 16;          // 8 per fixed tile
 // MMA issuers: warp 1 for fixed tile A, warp 18 for tile B, so that one issuer's barrier
 // waits and commits overlap the other's MMAs in the tensor pipe
 constexpr int kMmaWarpB = kEpiWarp0 + kEpiWarps;
@@ -63,9 +69,12 @@ constexpr int kAccCols = 128;
 constexpr int kAccBufs = 2;            // accumulator pairs in TMEM (kAccBufs x 2 x 128 columns)
 constexpr int kSched = 4;              // depth of the item-index ring (producer -> consumers)
 // Column-sum mode: the lse values of each streamed query tile reach shared memory by
-// TMA, in a ring of their own that the epilogue releases (plain loads from the epilogue
+// TMA, in a ring of their own that the normaliser warp releases (plain loads from there
 // queue behind the tile stream and stall it for several steps).
 constexpr int kLseSlots = 8;
+// Prepared normalisers: a step's are read after its accumulator's release, at the latest before
+// the release of the step after next, which the writer of the fourth step from it waits for.
+constexpr int kNlSlots = 4;
 constexpr int kLseBox = kTile + 4;     // floats per copy: the tile's 128, from a 16-byte boundary
 constexpr int kLseSlotBytes = 640;     // >= kLseBox * 4, multiple of 128
 
@@ -84,16 +93,21 @@ struct alignas(16) TcItem {
     int h, h2, g, kt, qt0, qt1, chunk;
 };
 
-template <int D>
+// Shared memory holds six tiles of d = 128.  The row normalisers' items are short (one query tile
+// of two heads) and their fixed tiles are double-buffered, with a ring of 2.  A column-sum item
+// streams dozens of tiles: one buffer of fixed tiles and a ring of 4 (16 prompts 118 -> 108 us,
+// 256 prompts 4.73 -> 4.66 ms; the same split takes the row normalisers from 106 to 114 us).
+template <int D, int MODE>
 struct Cfg {
     static constexpr int kAtoms = D / 64;
     static constexpr int kTileBytes = kTile * 128 * kAtoms;  // 128 rows x D bf16
-    static constexpr int kStages = D == 64 ? 6 : 2;
+    static constexpr int kFix = D == 128 && MODE == kModeImp ? 1 : 2;  // buffers of fixed tiles
+    static constexpr int kStages = D == 64 ? 6 : 6 - 2 * kFix;
     // dynamic smem layout (offsets from a 1024-aligned base)
-    static constexpr int kFixOff = 0;                               // [2 buffers][A, B]
-    static constexpr int kRingOff = 4 * kTileBytes;
-    static constexpr int kNlOff = kRingOff + kStages * kTileBytes;  // [kAccBufs][128] f32
-    static constexpr int kMergeOff = kNlOff + kAccBufs * kTile * 4;   // [2][A, B][4][32] float2
+    static constexpr int kFixOff = 0;                               // [kFix][A, B]
+    static constexpr int kRingOff = 2 * kFix * kTileBytes;
+    static constexpr int kNlOff = kRingOff + kStages * kTileBytes;  // [kNlSlots][128] f32
+    static constexpr int kMergeOff = kNlOff + kNlSlots * kTile * 4;   // [2][A, B][4][32] float2
     static constexpr int kBarOff = kMergeOff + 2 * 2 * 4 * 32 * 8;
     // fix_full/empty[2], ring_full/empty[kStages], acc_full/empty[A, B][kAccBufs],
     // drain[A, B], sched_full/empty[kSched], xfull/xempty[2][A, B][4], lse_full/empty[kLseSlots]
@@ -221,7 +235,7 @@ template <int D, int MODE>
 __global__ void __launch_bounds__(threads_of(MODE), 1)
     attn_tc_kernel(const __grid_constant__ CUtensorMap tm_fix, const __grid_constant__ CUtensorMap tm_str,
                    const __grid_constant__ CUtensorMap tm_lse, const TcArgs a) {
-    using C = Cfg<D>;
+    using C = Cfg<D, MODE>;
     extern __shared__ uint8_t smem_raw[];
     // an offset, not a rounded address: the compiler then knows the pointer as shared memory
     uint8_t* sm = smem_raw + (-smem_u32(smem_raw) & 1023u);
@@ -256,7 +270,7 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
         }
         for (int i = 0; i < 2 * kAccBufs; ++i) {
             mbar_init(&acc_full[i], MODE == kModeImp ? 2 : 1);  // the issuer; the normaliser warp
-            mbar_init(&acc_empty[i], MODE == kModeLse ? kEpiWarps / 2 : kEpiWarps / 4);  // its readers
+            mbar_init(&acc_empty[i], kEpiWarps / 2);  // its readers
         }
         for (int i = 0; i < C::kStages; ++i) {
             mbar_init(&ring_full[i], 1);
@@ -337,8 +351,8 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
                 sched_item[slot] = t;
                 mbar_arrive(&sched_full[slot]);  // release: the item is visible to waiters
                 if (item < 0) break;
-                const int fb = it & 1;
-                if (it >= 2 && !wait_bar(&fix_empty[fb], ((it >> 1) - 1) & 1, abort_flag, a.status, a.wait_cycles)) break;
+                const int fb = it % C::kFix;
+                if (it >= C::kFix && !wait_bar(&fix_empty[fb], ((it / C::kFix) - 1) & 1, abort_flag, a.status, a.wait_cycles)) break;
                 mbar_expect_tx(&fix_full[fb], 2 * C::kTileBytes);
 #pragma unroll
                 for (int tau = 0; tau < 2; ++tau)
@@ -399,8 +413,10 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
                     const uint32_t s2 = lse_issued - 1 - k;  // the last copy into each slot
                     drain_wait(&lse_full[s2 % kLseSlots], (s2 / kLseSlots) & 1, a.status);
                 }
-            for (int fb = 0; fb < 2 && fb < n_items; ++fb)
-                drain_wait(&fix_full[fb], (uint32_t)(((n_items - 1 - fb) / 2) & 1), a.status);
+            for (int k = 0; k < C::kFix && k < n_items; ++k) {
+                const int last = n_items - 1 - k;  // the last copy into each buffer
+                drain_wait(&fix_full[last % C::kFix], (uint32_t)((last / C::kFix) & 1), a.status);
+            }
         }
     } else if (warp == 1 || warp == kMmaWarpB) {
         // --------------------------------------------- MMA issuers (tile A, tile B)
@@ -411,8 +427,8 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
             for (int it = 0;; ++it) {
                 const TcItem t = consume_item(it, false);
                 if (!t.valid) break;
-                const int fb = it & 1;
-                if (!wait_bar(&fix_full[fb], (it >> 1) & 1, abort_flag, a.status, a.wait_cycles)) break;
+                const int fb = it % C::kFix;
+                if (!wait_bar(&fix_full[fb], (it / C::kFix) & 1, abort_flag, a.status, a.wait_cycles)) break;
                 const uint32_t fix_addr = smem_u32(fix + (fb * 2 + tau) * C::kTileBytes);
                 bool ok = true;
                 int q_it = t.qt0;  // column sums: the step's query tile
@@ -458,28 +474,29 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
     } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + kEpiWarps) {
         // ------------------------------------------------------------- epilogue
         const int e = warp - kEpiWarp0;
-        // LSE mode: warps 8 tau .. 8 tau + 7 read fixed tile tau at every step, two warps per
-        //   quarter, one per column half (sub).
-        // Column-sum mode: warps 4 g .. 4 g + 3 read fixed tile g & 1 at the steps of parity
-        //   sub = g >> 1 (all 128 columns), so that the groups of the two accumulator buffers
-        //   work a step apart and each step's lse values are read by 8 warps.
-        constexpr int kChunks = MODE == kModeLse ? 2 : 4;  // 32-column chunks per step
-        const int tau = MODE == kModeLse ? e >> 3 : (e >> 2) & 1;  // fixed tile: 0 = A, 1 = B
-        const int sub = MODE == kModeLse ? (e >> 2) & 1 : e >> 3;  // which of a row's two partials
-        const int col0 = MODE == kModeLse ? sub * 64 : 0;
+        // warps 8 tau .. 8 tau + 7 read fixed tile tau at every step, two warps per quarter of its
+        // rows, one per column half (sub)
+        const int tau = e >> 3;                    // fixed tile: 0 = A, 1 = B
+        const int sub = (e >> 2) & 1;              // which of a row's two partials
+        const int col0 = sub * 64;
         const int q = warp & 3;                    // TMEM lane quarter
         const int row = q * 32 + lane;             // accumulator row owned by this thread
         uint32_t step = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
-            const TcItem t = consume_item(it, true);
+            // the item stays in its slot until its end: what only the end needs takes no registers
+            if (!warp_wait(&sched_full[it % kSched], (uint32_t)((it / kSched) & 1), abort_flag, a.status, a.wait_cycles))
+                break;
+            const TcItem& t = sched_item[it % kSched];
             if (!t.valid) break;
+            const int n_steps = t.n_steps, kt = t.kt + tau, my_qt = t.qt0 + tau * t.dq;
+            const int qt0 = t.qt0, qt1 = t.qt1;
             // column-sum mode: partial sums of this thread's four key rows 8 s + g8 (s = 0..3)
             // of the quarter, over its columns (16x256b layout, see below)
             float2 acc4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f),
                               make_float2(0.f, 0.f)};
             float m = -1e30f, ssum = 0.f;          // LSE mode
-            int qt = t.qt0;                        // column sums: the step's query tile
+            int qt = qt0;                          // column sums: the step's query tile
             auto do_step = [&](int s) -> bool {
                 const int ab = (int)(step % kAccBufs);
                 const int abar = tau * kAccBufs + ab;  // accumulator barrier
@@ -487,130 +504,106 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
                     return false;
                 tc_fence_after();
                 // column-sum mode: this warp's key tile against the streamed query tile
-                const int kt = t.kt + tau;
                 const bool imp_skip = MODE == kModeImp && qt < kt;   // queries all before keys
                 const bool imp_diag = MODE == kModeImp && qt == kt;
                 // LSE mode: this warp's query tile against streamed key tile s
-                const int my_qt = t.qt0 + tau * t.dq;
                 const bool lse_skip = MODE == kModeLse && s > my_qt;  // keys all after queries
                 const bool lse_diag = MODE == kModeLse && s == my_qt;
-                if (imp_skip || lse_skip) {  // nothing to read: hand the accumulator back
+                auto release = [&]() {  // hand the accumulator back, before any arithmetic on it
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&acc_empty[abar]);
+                };
+                if (imp_skip || lse_skip) {  // nothing to read
+                    release();
                     return true;
                 }
                 const uint32_t taddr =
                     tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((ab * 2 + tau) * kAccCols + col0);
                 const float2 sc = make_float2(a.scale_log2, a.scale_log2);
                 if constexpr (MODE == kModeImp) {
-                    const float* nl = nl_all + ab * kTile;  // -log2e * lse of the step's query columns
+                    const float* nl = nl_all + (step % kNlSlots) * kTile;  // -log2e * lse of the query columns
                     // 16x256b loads: thread (g8, c4) = (lane / 4, lane % 4) holds key rows
-                    // q*32 + 16 lh + 8 jj + g8 and query columns 64 h + 8 k + 2 c4 + {0, 1}.
+                    // q*32 + 16 lh + 8 jj + g8 and query columns col0 + 8 k + 2 c4 + {0, 1}.
                     // Each query column's -lse log2e is then needed by 8 lanes only: 8
-                    // two-float shared loads per 64 columns, each one wavefront, instead of
-                    // every lane reading all 128 values (the shared-memory pipe was the bound).
+                    // two-float shared loads, each one wavefront, instead of every lane
+                    // reading all 64 values (the shared-memory pipe was the bound).
                     const int g8 = lane >> 2, c4 = lane & 3;
+                    uint32_t raw[2][32];
+                    tmem_ld16x256_x8(taddr, raw[0]);
+                    tmem_ld16x256_x8(taddr + (16u << 16), raw[1]);
+                    tmem_wait_ld();
+                    tie32(raw[0]);
+                    tie32(raw[1]);
+                    release();
+                    auto add = [&](auto diag) {
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        float2 n2[8];
+                        for (int k = 0; k < 8; ++k) {
+                            const float2 n2 = *reinterpret_cast<const float2*>(nl + col0 + 8 * k + 2 * c4);
 #pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            n2[k] = *reinterpret_cast<const float2*>(nl + h * 64 + 8 * k + 2 * c4);
-#pragma unroll
-                        for (int lh = 0; lh < 2; ++lh) {
-                            uint32_t raw[32];
-                            tmem_ld16x256_x8(taddr + ((uint32_t)(16 * lh) << 16) + (uint32_t)(h * 64), raw);
-                            tmem_wait_ld();
-                            if (h == 1 && lh == 1) {  // all 128 columns read: release the accumulator
-                                tc_fence_before();
-                                __syncwarp();
-                                if (lane == 0) mbar_arrive(&acc_empty[abar]);
-                            }
-                            if (!imp_diag) {
-#pragma unroll
-                                for (int k = 0; k < 8; ++k) {
-                                    const float2 x0 = __ffma2_rn(
-                                        make_float2(__uint_as_float(raw[4 * k]), __uint_as_float(raw[4 * k + 1])),
-                                        sc, n2[k]);
-                                    const float2 x1 = __ffma2_rn(
-                                        make_float2(__uint_as_float(raw[4 * k + 2]), __uint_as_float(raw[4 * k + 3])),
-                                        sc, n2[k]);
-                                    acc4[2 * lh] = __fadd2_rn(acc4[2 * lh], make_float2(ex2(x0.x), ex2(x0.y)));
-                                    acc4[2 * lh + 1] = __fadd2_rn(acc4[2 * lh + 1], make_float2(ex2(x1.x), ex2(x1.y)));
+                            for (int r4 = 0; r4 < 4; ++r4) {
+                                const uint32_t* w = raw[r4 >> 1] + 4 * k + 2 * (r4 & 1);
+                                const float2 x = __ffma2_rn(
+                                    make_float2(__uint_as_float(w[0]), __uint_as_float(w[1])), sc, n2);
+                                float2 p = make_float2(ex2(x.x), ex2(x.y));
+                                if (decltype(diag)::value) {  // query i0 = column, key j = row; keep i0 >= j
+                                    const int i0 = col0 + 8 * k + 2 * c4 - a.exclude_self;
+                                    const int j = q * 32 + 8 * r4 + g8;
+                                    p.x = i0 >= j ? p.x : 0.f;
+                                    p.y = i0 + 1 >= j ? p.y : 0.f;
                                 }
-                            } else {  // diagonal tile: query i = column, key j = row; keep i >= j
-#pragma unroll
-                                for (int k = 0; k < 8; ++k) {
-#pragma unroll
-                                    for (int jj = 0; jj < 2; ++jj) {
-                                        const float2 x = __ffma2_rn(
-                                            make_float2(__uint_as_float(raw[4 * k + 2 * jj]),
-                                                        __uint_as_float(raw[4 * k + 2 * jj + 1])),
-                                            sc, n2[k]);
-                                        const int i0 = h * 64 + 8 * k + 2 * c4;
-                                        const int j = q * 32 + 16 * lh + 8 * jj + g8;
-                                        const bool k0 = a.exclude_self ? i0 > j : i0 >= j;
-                                        const bool k1 = a.exclude_self ? i0 + 1 > j : i0 + 1 >= j;
-                                        acc4[2 * lh + jj] = __fadd2_rn(
-                                            acc4[2 * lh + jj], make_float2(k0 ? ex2(x.x) : 0.f, k1 ? ex2(x.y) : 0.f));
-                                    }
-                                }
+                                acc4[r4] = __fadd2_rn(acc4[r4], p);
                             }
                         }
-                    }
+                    };
+                    if (imp_diag) add(std::true_type{});
+                    else add(std::false_type{});
                     return true;
                 } else {
-                // LSE mode: chunks of 32 columns of this thread's query row: load, (release the
-                // accumulator after the last), reduce
+                // LSE mode: 64 columns of this thread's query row
+                float v[64];
+                tmem_ld32(taddr, v);
+                tmem_ld32(taddr + 32, v + 32);
+                tmem_wait_ld();
+                tie32(v);
+                tie32(v + 32);
+                release();
+                if (lse_diag) {  // diagonal tile: keys j = col after the query i = row
 #pragma unroll
-                for (int ch = 0; ch < kChunks; ++ch) {
-                    float v[32];
-                    tmem_ld32(taddr + ch * 32, v);
-                    tmem_wait_ld();
-                    if (ch == kChunks - 1) {
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&acc_empty[abar]);
-                    }
-                    const int cb = col0 + ch * 32;  // tile column of v[0]
-                    {
-                        if (lse_diag) {  // diagonal tile: keys j = col after the query i = row
-#pragma unroll
-                            for (int c = 0; c < 32; ++c)
-                                if (cb + c > row) v[c] = -INFINITY;
-                        }
-                        // chunk max: four independent 3-input max chains, then a short tree
-                        float mk[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const float* w8 = v + 8 * k;
-                            mk[k] = fmaxf(fmax3(fmax3(w8[0], w8[1], w8[2]), w8[3], w8[4]),
-                                          fmax3(w8[5], w8[6], w8[7]));
-                        }
-                        const float mx = fmaxf(fmax3(mk[0], mk[1], mk[2]), mk[3]);
-                        const float nm = fmaxf(m, mx * a.scale_log2);
-                        ssum *= ex2(m - nm);
-                        m = nm;
-                        const float2 nm2 = make_float2(-nm, -nm);
-                        float2 s2[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f),
-                                        make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-                        for (int c = 0; c < 32; c += 2) {
-                            float2 x = __ffma2_rn(make_float2(v[c], v[c + 1]), sc, nm2);
-                            s2[(c >> 1) & 3] = __fadd2_rn(s2[(c >> 1) & 3], make_float2(ex2(x.x), ex2(x.y)));
-                        }
-                        const float2 s01 = __fadd2_rn(s2[0], s2[1]), s23 = __fadd2_rn(s2[2], s2[3]);
-                        const float2 st = __fadd2_rn(s01, s23);
-                        ssum += st.x + st.y;
-                    }
+                    for (int c = 0; c < 64; ++c)
+                        if (col0 + c > row) v[c] = -INFINITY;
                 }
+                // max: four independent 3-input max chains, then a short tree
+                float mk[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float* w = v + 16 * k;
+                    float x = fmax3(w[0], w[1], w[2]);
+#pragma unroll
+                    for (int c = 3; c < 15; c += 2) x = fmax3(x, w[c], w[c + 1]);
+                    mk[k] = fmaxf(x, w[15]);
+                }
+                const float nm = fmaxf(m, fmaxf(fmax3(mk[0], mk[1], mk[2]), mk[3]) * a.scale_log2);
+                ssum *= ex2(m - nm);
+                m = nm;
+                const float2 nm2 = make_float2(-nm, -nm);
+                float2 s2[4];
+#pragma unroll
+                for (int c = 0; c < 64; c += 2) {
+                    const float2 x = __ffma2_rn(make_float2(v[c], v[c + 1]), sc, nm2);
+                    const float2 p = make_float2(ex2(x.x), ex2(x.y));
+                    float2& d = s2[(c >> 1) & 3];
+                    d = c < 8 ? p : __fadd2_rn(d, p);
+                }
+                const float2 st = __fadd2_rn(__fadd2_rn(s2[0], s2[1]), __fadd2_rn(s2[2], s2[3]));
+                ssum += st.x + st.y;
                 return true;
                 }
             };
-            for (int s = 0; s < t.n_steps; ++s, ++step) {
-                if ((MODE == kModeLse || (int)(step & 1) == sub) && !(ok = do_step(s))) break;
-                if (MODE == kModeImp && ++qt == t.qt1) qt = t.qt0;
+            for (int s = 0; s < n_steps; ++s, ++step) {
+                ok = do_step(s);
+                if (!ok) break;
+                if (MODE == kModeImp && ++qt == qt1) qt = qt0;
             }
             if (!ok) break;
             // column-sum mode: the four lanes c4 of a g8 hold columns of the same four rows;
@@ -666,12 +659,13 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
                         a.lse_out[(int64_t)h * a.sumT + t.t0 + i] = (mm + lg2(ss)) * kLn2;
                 }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sched_empty[it % kSched]);
         }
     } else if (MODE == kModeImp && warp == kNlWarp) {
         // ------------------------------------------------------ row normalisers
         // -log2e * lse of every step's 128 query columns, -inf past the prompt, from the copied
-        // values to the buffer of the step's accumulators; the arrival on their barriers hands
-        // both over at once, and their release frees both.
+        // values to the step's slot; the arrival on the accumulators' barriers hands both over
         uint32_t step = 0;
         bool ok = true;
         for (int it = 0; ok; ++it) {
@@ -699,7 +693,7 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
                          warp_wait(&acc_empty[kAccBufs + ab], (use - 1) & 1, abort_flag, a.status, a.wait_cycles);
                 if (!ok) break;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) nl_all[ab * kTile + 32 * k + lane] = r[k];
+                for (int k = 0; k < 4; ++k) nl_all[(step % kNlSlots) * kTile + 32 * k + lane] = r[k];
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(&acc_full[ab]);
@@ -754,7 +748,7 @@ template <int D, int MODE>
 estp_status launch_tc(estp_ctx* ctx, const CUtensorMap& fixm, const CUtensorMap& strm,
                       const CUtensorMap& lsem, const TcArgs& a, cudaStream_t st) {
     auto kern = attn_tc_kernel<D, MODE>;
-    const int smem = Cfg<D>::kSmemBytes;
+    const int smem = Cfg<D, MODE>::kSmemBytes;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return cuda_fail(e, "tc kernel smem attribute");
     // a programmatic dependent of the plan kernel or of the row normalisers: the launch and the

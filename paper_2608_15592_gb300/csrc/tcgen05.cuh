@@ -114,6 +114,19 @@ __device__ __forceinline__ void tmem_wait_ld() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Orders every later use of r[0..31] after the asm statements before it (the wait for the load
+// that fills them): to the compiler the load's results are plain registers.
+template <class T>
+__device__ __forceinline__ void tie32(T* r) {
+    static_assert(sizeof(T) == 4, "32-bit registers");
+#pragma unroll
+    for (int k = 0; k < 32; k += 8) {
+        uint32_t* w = reinterpret_cast<uint32_t*>(r) + k;
+        asm volatile("" : "+r"(w[0]), "+r"(w[1]), "+r"(w[2]), "+r"(w[3]), "+r"(w[4]), "+r"(w[5]),
+                          "+r"(w[6]), "+r"(w[7]));
+    }
+}
+
 // The driver's cuTensorMapEncodeTiled, looked up once (NULL when unavailable).
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 

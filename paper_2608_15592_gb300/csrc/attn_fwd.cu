@@ -441,7 +441,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int q = warp & 3;                // TMEM lane quarter
         const int grp = (e >> 2) & 1;          // takes the steps of this parity
         const int half = e >> 3;               // 64-column half of S / P and of O's columns
-        const int row = q * 32 + lane;         // query row of the tile owned by this thread
         const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16);
         // S / P layout (16x256b / 16x128b): thread (g, c) = (lane / 4, lane % 4) holds rows
         // 32q + g + 8r, r = 0..3, and key columns 8k + 2c + 0..1, k = 0..7, of its half
@@ -451,8 +450,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int it = 0; ok; ++it) {
             const FwdItem t = consume_item(it, true);
             if (!t.valid) break;
-            const int i_loc = t.qt * kT + row;                 // query index in the prompt
-            const bool valid = i_loc < t.T;
             // the row normalisers (log2 units) of the 4 rows of the S / P layout; a row past
             // the prompt gets +inf, so its probabilities are exactly 0
             float lr[4];
@@ -546,27 +543,52 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             if (!ok) break;
             if ((int)((step - 1) & 1) != grp) continue;  // the other group ends this item
-            // O of the item: this warp's 32 rows x 64 columns
+            // O of the item: this warp's 32 rows x 64 columns, in the layout of S (lane (g8, c4)
+            // holds columns 8k + 2 c4 + 0..1 of rows g8 + 8r), released before it is stored
             if (!warp_wait(&o_full[grp], n_out & 1, abort_flag, a.status, a.wait_cycles)) break;
             ++n_out;
             tc_fence_after();
-#pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {
-                float v[32];
-                tmem_ld32(lane_base + kColO + half * 64 + ch * 32, v);
-                tmem_wait_ld();
-                if (valid && in_bounds(t.t0 + i_loc < a.sumT && t.h >= 0 && t.h < a.Hq, a.status)) {
-                    uint4* out = reinterpret_cast<uint4*>(
-                        a.O + ((t.t0 + i_loc) * a.Hq + t.h) * (int64_t)kD + half * 64 + ch * 32);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        out[k] = make_uint4(pack_bf16(v[8 * k], v[8 * k + 1]), pack_bf16(v[8 * k + 2], v[8 * k + 3]),
-                                            pack_bf16(v[8 * k + 4], v[8 * k + 5]), pack_bf16(v[8 * k + 6], v[8 * k + 7]));
-                }
-            }
+            uint32_t o[2][32];
+            tmem_ld16x256_x8(lane_base + kColO + half * 64, o[0]);
+            tmem_ld16x256_x8(lane_base + (16u << 16) + kColO + half * 64, o[1]);
+            tmem_wait_ld();
+            tie32(o[0]);
+            tie32(o[1]);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(o_empty);
+            // The four lanes of a g8 turn their 4 x 4 blocks of column pairs, so that each holds 16
+            // bytes of a row and a store covers 64 bytes of 8 rows (a row per lane would touch 32
+            // cache lines a store)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const int i_loc = t.qt * kT + q * 32 + g8 + 8 * r;  // query index in the prompt
+                uint4* out = reinterpret_cast<uint4*>(
+                    a.O + ((t.t0 + i_loc) * a.Hq + t.h) * (int64_t)kD + half * 64);
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    uint32_t u[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const uint32_t* w = o[r >> 1] + 4 * (4 * m + k) + 2 * (r & 1);
+                        u[k] = pack_bf16(__uint_as_float(w[0]), __uint_as_float(w[1]));
+                    }
+                    // block (lane c, k) -> (lane k, c): first the 2 x 2 corners, then inside them
+#pragma unroll
+                    for (int bit = 2; bit > 0; bit >>= 1) {
+                        const bool hi = (c4 & bit) != 0;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            if (k & bit) continue;
+                            const uint32_t got = __shfl_xor_sync(0xffffffffu, hi ? u[k] : u[k | bit], bit);
+                            if (hi) u[k] = got;
+                            else u[k | bit] = got;
+                        }
+                    }
+                    if (i_loc < t.T && in_bounds(t.t0 + i_loc < a.sumT && t.h >= 0 && t.h < a.Hq, a.status))
+                        out[4 * m + c4] = make_uint4(u[0], u[1], u[2], u[3]);
+                }
+            }
         }
     }
     tc_fence_before();

@@ -119,6 +119,10 @@ struct Cfg {
     static constexpr int kMiscOff = (kBarOff + kNumBars * 8 + 15) / 16 * 16;
     static constexpr int kLseOff = (kMiscOff + 16 + (int)sizeof(TcItem) * kSched + 127) / 128 * 128;  // lse ring
     static constexpr int kSmemBytes = kLseOff + kLseSlots * kLseSlotBytes + 1024;  // + alignment slack
+    // the items are copied whole, in accesses of up to 16 bytes, and the normalisers read in pairs
+    static_assert(alignof(TcItem) == 16 && sizeof(TcItem) % 16 == 0 && kMiscOff % 16 == 0, "item alignment");
+    static_assert(kBarOff % 8 == 0 && kNlOff % 16 == 0 && kMergeOff % 8 == 0 && kLseOff % 128 == 0, "alignment");
+    static_assert(kSmemBytes <= 227 * 1024, "shared memory per CTA");
 };
 
 struct TcArgs {

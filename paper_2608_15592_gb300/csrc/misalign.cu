@@ -15,10 +15,12 @@
 // index below which they do, in the same way.  A last pass counts the two intersections.
 // Integer counts: the result is exact.
 //
-// What bounds it is latency: each pass is one read of the prompt (from L1 after the first),
-// three barriers and a scan.  256 prompts of 128 to 4096 tokens: 144 -> 22.5 us a call; four
-// prompts of 32768: 234 -> 129 us.  (Before: 32 passes of 8-bit digits, one selection at a time,
-// each scanned by one thread.)
+// What bounds it is latency: each pass is one look at the prompt's keys (those of its first 2048
+// tokens in registers, the rest from L1), three barriers and a scan.  While the two intervals of a
+// value agree, which they do in the first pass, one histogram serves both: half of the shared
+// atomics.  256 prompts of 128 to 4096 tokens: 144 us for 32 passes of 8-bit digits, one selection
+// at a time, each scanned by one thread; 23.0 for the passes above with every key re-read and four
+// histograms; 17.0 now.  Four prompts of 32768: 234, 127 and 65 us.
 #include "estp_internal.cuh"
 
 namespace estp {
@@ -30,6 +32,9 @@ constexpr int kBins = 1024;
 constexpr int kBinBits = 10;
 constexpr int kGroup = kThreads / kSel;   // threads that scan one selection's histogram
 constexpr int kPerThread = kBins / kGroup;
+// Tokens a thread keeps in registers.  256 prompts of up to 4096 tokens 18.8 / 17.0 / 16.6 us and 16
+// short ones 10.9 / 8.5 / 9.9 with 1 / 4 / 8.
+constexpr int kCached = 4;
 
 // monotone map float -> uint32 (larger float, larger image); inputs are finite, and
 // -0 maps with +0 (they are equal values, so their order falls to the index)
@@ -59,11 +64,13 @@ struct Shared {
     int n_hl, n_lh;
 };
 
-// Narrows every selection (those with rank > 0) to a single key; key(s, i) is token i's key in
-// selection s, and in(s, i) whether it takes part.  All threads call; sh.sel is read and
-// written between barriers.
-template <typename Key, typename In>
-__device__ __forceinline__ void narrow(Shared& sh, int T, Key key, In in) {
+// Narrows every selection (those with rank > 0) to a single key.  each(f) calls f(i, kh, ks) for
+// this thread's tokens with the keys of H and S; key(s, i, kh, ks) is a token's key in selection
+// s, and in(s, i, kh, ks) whether it takes part.  kTwins: the two selections of one value see the
+// same keys, so that while their intervals agree one histogram serves both.  All threads call;
+// sh.sel is read and written between barriers.
+template <bool kTwins, typename Each, typename Key, typename In>
+__device__ __forceinline__ void narrow(Shared& sh, Each each, Key key, In in) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int grp = threadIdx.x / kGroup;  // the selection this thread scans
     int shift[kSel];  // -1: done (every round takes kBinBits off, so at most four follow)
@@ -75,20 +82,24 @@ __device__ __forceinline__ void narrow(Shared& sh, int T, Key key, In in) {
 #pragma unroll
         for (int s = 0; s < kSel; ++s) lo[s] = sh.sel[s].lo;
         const Select mine = sh.sel[grp];
+        const bool twin[2] = {kTwins && lo[0] == lo[1] && shift[0] == shift[1],
+                              kTwins && lo[2] == lo[3] && shift[2] == shift[3]};
+        const int hist_of = twin[grp >> 1] ? grp & ~1 : grp;
         __syncthreads();
-        for (int i = threadIdx.x; i < T; i += kThreads)
+        each([&](int i, uint32_t kh, uint32_t ks) {
 #pragma unroll
             for (int s = 0; s < kSel; ++s)
-                if (shift[s] >= 0 && in(s, i)) {
-                    const uint32_t x = key(s, i), bin = (x - lo[s]) >> shift[s];
+                if (shift[s] >= 0 && !((s & 1) && twin[s >> 1]) && in(s, i, kh, ks)) {
+                    const uint32_t x = key(s, i, kh, ks), bin = (x - lo[s]) >> shift[s];
                     if (x >= lo[s] && bin < (uint32_t)kBins) atomicAdd(&sh.hist[s][bin], 1u);
                 }
+        });
         __syncthreads();
         // scan of the selection's bins: kPerThread a thread, its warp, its group's warps
         int cnt[kPerThread], sum = 0;
 #pragma unroll
         for (int j = 0; j < kPerThread; ++j) {
-            cnt[j] = (int)sh.hist[grp][(threadIdx.x % kGroup) * kPerThread + j];
+            cnt[j] = (int)sh.hist[hist_of][(threadIdx.x % kGroup) * kPerThread + j];
             sum += cnt[j];
         }
         int inc = sum;
@@ -121,7 +132,7 @@ __device__ __forceinline__ void narrow(Shared& sh, int T, Key key, In in) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads) misalign_kernel(const float* __restrict__ H,
+__global__ void __launch_bounds__(kThreads, 2) misalign_kernel(const float* __restrict__ H,
                                                             const float* __restrict__ S,
                                                             const int32_t* __restrict__ cu, int B,
                                                             int64_t sumT, int pct,
@@ -150,16 +161,31 @@ __global__ void __launch_bounds__(kThreads) misalign_kernel(const float* __restr
     }
     const float* h = H + t0;
     const float* s = S + t0;
-    auto val = [&](int sel, int i) { return ordered(sel < 2 ? h[i] : s[i]); };
+    // a thread's tokens: the keys of the first kCached stay in registers
+    uint32_t ch[kCached], cs[kCached];
+#pragma unroll
+    for (int j = 0; j < kCached; ++j) {
+        const int i = threadIdx.x + j * kThreads;
+        ch[j] = i < T ? ordered(h[i]) : 0u;
+        cs[j] = i < T ? ordered(s[i]) : 0u;
+    }
+    auto each = [&](auto f) {
+#pragma unroll
+        for (int j = 0; j < kCached; ++j) {
+            const int i = threadIdx.x + j * kThreads;
+            if (i < T) f(i, ch[j], cs[j]);
+        }
+        for (int i = threadIdx.x + kCached * kThreads; i < T; i += kThreads) f(i, ordered(h[i]), ordered(s[i]));
+    };
+    auto val = [](int sel, int, uint32_t kh, uint32_t ks) { return sel < 2 ? kh : ks; };
     // the spans of the prompt's keys
     uint32_t lo_h = 0xFFFFFFFFu, hi_h = 0, lo_s = 0xFFFFFFFFu, hi_s = 0;
-    for (int i = threadIdx.x; i < T; i += kThreads) {
-        const uint32_t kh = ordered(h[i]), ks = ordered(s[i]);
+    each([&](int, uint32_t kh, uint32_t ks) {
         lo_h = min(lo_h, kh);
         hi_h = max(hi_h, kh);
         lo_s = min(lo_s, ks);
         hi_s = max(hi_s, ks);
-    }
+    });
     lo_h = __reduce_min_sync(0xffffffffu, lo_h);
     hi_h = __reduce_max_sync(0xffffffffu, hi_h);
     lo_s = __reduce_min_sync(0xffffffffu, lo_s);
@@ -183,7 +209,7 @@ __global__ void __launch_bounds__(kThreads) misalign_kernel(const float* __restr
         sh.sel[threadIdx.x] = Select{lo, shift_for(hi - lo), (threadIdx.x & 1) ? k : T - k + 1, 0};
     }
     __syncthreads();
-    narrow(sh, T, val, [](int, int) { return true; });
+    narrow<true>(sh, each, val, [](int, int, uint32_t, uint32_t) { return true; });
     // Ties with a threshold: of its `equal` tokens the first n_take by index belong to the
     // group.  (Selected among the tied tokens' indices when that is not all of them.)
     uint32_t v[kSel];
@@ -197,19 +223,19 @@ __global__ void __launch_bounds__(kThreads) misalign_kernel(const float* __restr
         sh.sel[threadIdx.x] = Select{0, shift_for((uint32_t)T), take < r.equal ? take : 0, 0};
     }
     __syncthreads();
-    narrow(sh, T, [](int, int i) { return (uint32_t)i; }, [&](int q, int i) { return val(q, i) == v[q]; });
+    narrow<false>(sh, each, [](int, int i, uint32_t, uint32_t) { return (uint32_t)i; },
+                  [&](int q, int i, uint32_t kh, uint32_t ks) { return val(q, i, kh, ks) == v[q]; });
 #pragma unroll
     for (int q = 0; q < kSel; ++q) cut[q] = sh.sel[q].rank > 0 ? (int)sh.sel[q].lo : T;
     if (threadIdx.x == 0) sh.n_hl = sh.n_lh = 0;
     __syncthreads();
     int hl = 0, lh = 0;
-    for (int i = threadIdx.x; i < T; i += kThreads) {
-        const uint32_t kh = ordered(h[i]), ks = ordered(s[i]);
+    each([&](int i, uint32_t kh, uint32_t ks) {
         const bool th = kh > v[0] || (kh == v[0] && i <= cut[0]), bh = kh < v[1] || (kh == v[1] && i <= cut[1]);
         const bool ts = ks > v[2] || (ks == v[2] && i <= cut[2]), bs = ks < v[3] || (ks == v[3] && i <= cut[3]);
         hl += th && bs;
         lh += bh && ts;
-    }
+    });
     hl = __reduce_add_sync(0xffffffffu, hl);
     lh = __reduce_add_sync(0xffffffffu, lh);
     if (lane == 0) {

@@ -693,7 +693,7 @@ estp_status launch_attn_forward(estp_ctx* ctx, const void* Q, const void* K, con
     PlanInfo* info = plan_info(ws + off_items, B);
     PlanInfo* info2 = plan_info(ws + off_slots, B);
     // plans: items (prompt, query tile, head), and the partial slots (tile pairs x heads)
-    const PlanReq items{kT, 1, Hq, 1, base, info}, slots{kT, 1, Hq, 2, base2, info2};
+    const PlanReq items{kT, 1, Hq, 1, base, info, 0}, slots{kT, 1, Hq, 2, base2, info2, 0};
     const float* lse = lse_in;
     if (lse_in) {
         launch_plans(ctx, cu, B, sumT, max_seqlen, st, items, slots);

@@ -19,8 +19,8 @@ namespace estp {
 
 // One plan, computed by all 1024 threads of the calling block.
 static __device__ void plan_body(const int32_t* cu, int B, int64_t sumT, int max_seqlen, int tile,
-                                 int qc, int mult, int kind, int32_t* base, PlanInfo* info,
-                                 int* status) {
+                                 int qc, int mult, int kind, bool sorted, int32_t* base,
+                                 PlanInfo* info, int* status) {
     // thread t owns prompts [t*per, (t+1)*per); one read of cu, warp-shuffle scans
     __shared__ int64_t warp_sum[32];
     __shared__ int bad;
@@ -28,10 +28,23 @@ static __device__ void plan_body(const int32_t* cu, int B, int64_t sumT, int max
     if (tid == 0) bad = 0;
     __syncthreads();
     if (tid == 0 && (cu[0] != 0 || (int64_t)cu[B] != sumT)) bad = 1;
+    // a sorted plan's prompts by rank of length (equal lengths as they come)
+    __shared__ int16_t order[kMaxSorted];
+    if (sorted && tid < B) {
+        const int32_t len = cu[tid + 1] - cu[tid];
+        int rank = 0;
+        for (int b = 0; b < B; ++b) {
+            const int32_t other = cu[b + 1] - cu[b];
+            rank += other > len || (other == len && b < tid);
+        }
+        order[rank] = info->order[rank] = (int16_t)tid;
+    }
+    if (sorted) __syncthreads();
     const int per = (B + 1023) / 1024;
     const int b0 = min(B, tid * per), b1 = min(B, b0 + per);
     int64_t local = 0;
-    for (int b = b0; b < b1; ++b) {
+    for (int i = b0; i < b1; ++i) {
+        const int b = sorted ? order[i] : i;
         const int32_t len = cu[b + 1] - cu[b];
         if (len < 0 || len > max_seqlen) { bad = 1; continue; }
         const int nt = (len + tile - 1) / tile;
@@ -58,8 +71,9 @@ static __device__ void plan_body(const int32_t* cu, int B, int64_t sumT, int max
     const int64_t total = warp_sum[31];
     const bool ok = !bad && total < INT32_MAX / 2;  // item indices stay 32-bit
     int64_t run = inc - local + (wid > 0 ? warp_sum[wid - 1] : 0);
-    for (int b = b0; b < b1; ++b) {
-        base[b] = ok ? (int32_t)run : 0;
+    for (int i = b0; i < b1; ++i) {
+        base[i] = ok ? (int32_t)run : 0;
+        const int b = sorted ? order[i] : i;
         const int32_t len = cu[b + 1] - cu[b];
         const int nt = (len + tile - 1) / tile;
         if (len >= 0) run += (int64_t)mult * plan_count(nt, qc, kind);
@@ -69,6 +83,7 @@ static __device__ void plan_body(const int32_t* cu, int B, int64_t sumT, int max
         info->ok = ok ? 1 : 0;
         info->total = ok ? (int32_t)total : 0;
         info->next = 0;
+        info->sorted = sorted ? 1 : 0;
     }
     if (tid == 0 && !ok) report(status, ESTP_ERR_INVALID_ARG);
 }
@@ -80,7 +95,7 @@ __global__ void __launch_bounds__(1024) attn_plan_kernel(const int32_t* cu, int 
     // it waits for this grid before its first read of the plan
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const PlanReq p = plans.plan[blockIdx.x];
-    plan_body(cu, B, sumT, max_seqlen, p.tile, p.qc, p.mult, p.kind, p.base, p.info, status);
+    plan_body(cu, B, sumT, max_seqlen, p.tile, p.qc, p.mult, p.kind, p.sorted != 0, p.base, p.info, status);
 }
 
 namespace {
@@ -91,15 +106,17 @@ namespace {
 // where 128 would leave SMs idle), its streamed side comes in tiles of 128, and whatever of a
 // tile is wholly masked (above the diagonal, past the prompt) is left out in units of 64.
 // The bound is the FMA pipe (54 packed FMAs a clock and SM): a 128 x 128 tile takes 32 packed
-// FMAs a thread for four 16-byte shared loads.  Items come from a counter, the longest of a
-// prompt first.  4 prompts of 300 to 1500 tokens, 16 heads, d 128: row normalisers 485 -> 173 us,
-// column sums 857 -> 162 us against 64 x 64 tiles of scalar FMAs (4 x 4 a thread).
+// FMAs a thread for four 16-byte shared loads.  Items come from a counter, the longest prompt's
+// first and its longest first: with prompts in batch order the long items of a late prompt ended
+// alone (row normalisers 174 -> 158 us on 4 prompts, column sums 504 -> 369 on 32).  4 prompts of 300
+// to 1500 tokens, 16 heads, d 128, against 64 x 64 tiles of scalar FMAs (4 x 4 a thread): row
+// normalisers 485 -> 158 us, column sums 857 -> 162.
 constexpr int kFThreads = 256;
 constexpr int kFCols = 128;          // rows of a streamed tile
-// Items per SM below which the split gets finer.  Row normalisers at 3.2 items of 128 rows per
-// SM: 173 us with 128 rows, 183 with 64.  Column sums there: 243 us at 2 items per SM, 162 at 4
-// or 8, 234 at 16.
-constexpr int kFLseItemsPerSm = 3, kFImpItemsPerSm = 4;
+// Items per SM below which the split gets finer.  4 prompts of 300 to 1500 tokens, 16 heads, d 128
+// (2.5 items of 128 rows per SM): row normalisers 158 us with 128 rows, 171 with 64.  Column sums at
+// 4 and at 8 items per SM: 164 and 162 us there, 432 and 369 on 32 prompts of 100 to 1000.
+constexpr int kFLseItemsPerSm = 2, kFImpItemsPerSm = 8;
 
 template <int TM, int TN>
 using ScoreTile = SgemmTile<TM, TN, 16, true, true, false>;
@@ -117,6 +134,7 @@ struct F32Args {
     float scale_log2;          // softmax_scale * log2(e)
     ImpHeads hs;
     int exclude_self;
+    int sms;                   // SMs of the device (a block of each wave on every one)
     int qc;                    // column sums: query tiles per item
     float* part;               // column sums: [c_max][n_groups][sumT]
     float* lse_out;            // row normalisers: [Hq, sumT]
@@ -124,7 +142,14 @@ struct F32Args {
     int* status;
 };
 
-// Items of a block: its own index first, then the plan's counter.
+// First item of a block.  Items get shorter, so the second block of each SM takes them in the
+// reverse order: the SM with the longest first item gets the shortest second one.
+__device__ __forceinline__ int first_item(int sms) {
+    const int wave = blockIdx.x / sms, r = blockIdx.x - wave * sms;
+    return wave * sms + ((wave & 1) ? sms - 1 - r : r);
+}
+
+// The items after it come from the plan's counter.
 __device__ __forceinline__ int next_item(PlanInfo* info, int* slot) {
     __syncthreads();
     if (threadIdx.x == 0) *slot = (int)gridDim.x + atomicAdd(&info->next, 1);
@@ -140,8 +165,9 @@ __global__ void __launch_bounds__(kFThreads, TM == 8 ? 1 : 2) lse_f32_kernel(con
     constexpr int kRows = 16 * TM;
     const int total = a.info->total;
     const int rep = a.Hq / a.Hkv;
-    for (int item = blockIdx.x; item < total; item = next_item(a.info, &slot)) {
-        const LseItem it = decode_lse_item(item, a.base, a.B, a.cu, kRows, a.hs.n_heads);
+    for (int item = first_item(a.sms); item < total; item = next_item(a.info, &slot)) {
+        const int at = upper_slot(a.base, a.B, item);
+        const LseItem it = decode_lse_item_at(item, at, prompt_of(a.info, at), a.base, a.cu, kRows, a.hs.n_heads);
         const int h = a.hs.head_list[it.hslot];
         const int q0 = it.qt * kRows;
         const GemmSide qs{a.Q + (it.t0 * a.Hq + h) * a.d, (int64_t)a.Hq * a.d, it.T, 1};
@@ -214,8 +240,9 @@ __global__ void __launch_bounds__(kFThreads, 2) imp_f32_kernel(const F32Args a) 
     __shared__ int slot;
     constexpr int kRows = 16 * TM;
     const int total = a.info->total;
-    for (int item = blockIdx.x; item < total; item = next_item(a.info, &slot)) {
-        const ImpItem it = decode_imp_item(item, a.base, a.B, a.cu, kRows, a.qc);
+    for (int item = first_item(a.sms); item < total; item = next_item(a.info, &slot)) {
+        const int at = upper_slot(a.base, a.B, item);
+        const ImpItem it = decode_imp_item_at(item, at, prompt_of(a.info, at), a.base, a.cu, kRows, a.qc);
         const int k0 = it.kt * kRows;
         const int i_end = min(it.T, it.qt1 * kRows);  // queries of the item
         const GemmSide ks{a.K + (it.t0 * a.Hkv + a.hs.group[it.g]) * a.d, (int64_t)a.Hkv * a.d, it.T, 1};
@@ -362,6 +389,10 @@ int f32_rows(int B, int64_t sumT, int n_heads, int num_sms) {
     return (int64_t)B * n_heads * mean_tiles(B, sumT, 128) >= (int64_t)kFLseItemsPerSm * num_sms ? 128 : 64;
 }
 
+// Whether a plan sorts its prompts: where some items wait for others to end.  (Below that the
+// sorting and the look-up cost ~2 us and give nothing.)
+int f32_sorted(int B, int64_t items, int64_t blocks) { return B > 1 && B <= kMaxSorted && items > blocks; }
+
 F32Split f32_split(int B, int64_t sumT, const ImpHeads& hs, int num_sms) {
     F32Split s{128, 8, false};
     auto enough = [&] {
@@ -387,7 +418,8 @@ ImpHeads heads_apart(const ImpHeads& hs, int rep) {
 }
 
 template <class Kernel>
-cudaError_t launch_f32(estp_ctx* ctx, Kernel kernel, const F32Args& a, cudaStream_t st) {
+cudaError_t launch_f32(estp_ctx* ctx, Kernel kernel, F32Args& a, cudaStream_t st) {
+    a.sms = ctx->num_sms;
     int occ = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kFThreads, 0);
     if (e != cudaSuccess) return e;
@@ -397,7 +429,9 @@ cudaError_t launch_f32(estp_ctx* ctx, Kernel kernel, const F32Args& a, cudaStrea
 
 PlanReq lse_plan_f32(const ImpHeads& hs, int B, int64_t sumT, int num_sms, int32_t* base,
                      PlanInfo* info) {
-    return {f32_rows(B, sumT, hs.n_heads, num_sms), 1, hs.n_heads, 1, base, info};
+    const int rows = f32_rows(B, sumT, hs.n_heads, num_sms);
+    return {rows, 1, hs.n_heads, 1, base, info,
+            f32_sorted(B, (int64_t)B * hs.n_heads * mean_tiles(B, sumT, rows), rows == 128 ? num_sms : 2 * num_sms)};
 }
 
 // Row normalisers of the selected heads (fp32).
@@ -462,7 +496,9 @@ estp_status launch_importance(estp_ctx* ctx, const void* Q, const void* K, estp_
     int32_t* base = plan_base(ws + off_plan);
     PlanInfo* info = plan_info(ws + off_plan, B);
     float* part = reinterpret_cast<float*>(ws + off_part);
-    const PlanReq plan{tile, qc, hs.n_groups, 0, base, info};
+    const PlanReq plan{tile, qc, hs.n_groups, 0, base, info,
+                       tc ? 0 : f32_sorted(B, (int64_t)B * hs.n_groups * items_f(mean_tiles(B, sumT, tile), qc),
+                                           2 * ctx->num_sms)};
     float* lse_use = const_cast<float*>(lse);
     if (lse) {
         launch_plans(ctx, cu, B, sumT, max_seqlen, st, plan);

@@ -21,11 +21,14 @@ __host__ __device__ __forceinline__ int64_t items_f(int64_t n, int qc) {
     return (int64_t)qc * a * (a + 1) / 2 + r * (a + 1);
 }
 
+constexpr int kMaxSorted = 64;  // prompts of a plan in order of length
+
 struct PlanInfo {
     int32_t ok;      // 1 when cu_seqlens passed the device checks
     int32_t total;   // total items
     int32_t next;    // dynamic work counter of the persistent kernels (zeroed by the plan)
-    int32_t pad;
+    int32_t sorted;  // 1: items run over the prompts order[0], order[1], .. (longest first)
+    int16_t order[kMaxSorted];
 };
 
 // Per-prompt count of a plan of kind 0: importance items f(nt); kind 1: one per tile, nt;
@@ -34,11 +37,13 @@ __host__ __device__ __forceinline__ int64_t plan_count(int64_t nt, int qc, int k
     return kind == 0 ? items_f(nt, qc) : kind == 1 ? nt : nt * (nt + 1) / 2;
 }
 
-// One plan: each prompt counts mult * plan_count(ceil(length / tile), qc, kind) items.
+// One plan: each prompt counts mult * plan_count(ceil(length / tile), qc, kind) items.  sorted (at
+// most kMaxSorted prompts): the prompts run from the longest to the shortest.
 struct PlanReq {
     int tile, qc, mult, kind;
-    int32_t* base;   // [B + 1] prefix of the counts
+    int32_t* base;   // [B + 1] prefix of the counts, in the order of the prompts
     PlanInfo* info;
+    int sorted;
 };
 constexpr int kMaxPlans = 3;
 struct PlanSet {
@@ -71,8 +76,13 @@ struct ImpItem {
     int T;
 };
 
-// Item `item` of prompt b (the prompt whose items contain it: upper_slot(base, B, item)).
-__device__ __forceinline__ ImpItem decode_imp_item_at(int item, int b, const int32_t* base,
+// The prompt whose items start at base[slot], slot = upper_slot(base, B, item).
+__device__ __forceinline__ int prompt_of(const PlanInfo* info, int slot) {
+    return info->sorted ? info->order[slot] : slot;
+}
+
+// Item `item` of prompt b, whose items start at base[slot].
+__device__ __forceinline__ ImpItem decode_imp_item_at(int item, int slot, int b, const int32_t* base,
                                                       const int32_t* cu, int tile, int qc) {
     ImpItem it;
     it.b = b;
@@ -85,7 +95,7 @@ __device__ __forceinline__ ImpItem decode_imp_item_at(int item, int b, const int
         return (uint32_t)qc * (a * (a + 1) / 2) + r * (a + 1);
     };
     const uint32_t per_group = f((uint32_t)nt);
-    const uint32_t local = (uint32_t)(item - base[it.b]);
+    const uint32_t local = (uint32_t)(item - base[slot]);
     it.g = (int)(local / per_group);
     const uint32_t rem = local - (uint32_t)it.g * per_group;
     int lo = 0, hi = nt - 1;  // largest kt with F(kt) <= rem
@@ -100,9 +110,9 @@ __device__ __forceinline__ ImpItem decode_imp_item_at(int item, int b, const int
     return it;
 }
 
-__device__ __forceinline__ ImpItem decode_imp_item(int item, const int32_t* base, int B,
-                                                   const int32_t* cu, int tile, int qc) {
-    return decode_imp_item_at(item, upper_slot(base, B, item), base, cu, tile, qc);
+__device__ __forceinline__ ImpItem decode_imp_item_at(int item, int b, const int32_t* base,
+                                                      const int32_t* cu, int tile, int qc) {
+    return decode_imp_item_at(item, b, b, base, cu, tile, qc);
 }
 
 struct LseItem {
@@ -111,18 +121,23 @@ struct LseItem {
     int T;
 };
 
-__device__ __forceinline__ LseItem decode_lse_item_at(int item, int b, const int32_t* base,
+__device__ __forceinline__ LseItem decode_lse_item_at(int item, int slot, int b, const int32_t* base,
                                                       const int32_t* cu, int tile, int n_heads) {
     LseItem it;
     it.b = b;
     it.t0 = cu[it.b];
     it.T = cu[it.b + 1] - cu[it.b];
     const int nt = (it.T + tile - 1) / tile;
-    const int local = item - base[it.b];
+    const int local = item - base[slot];
     const int rank = local / n_heads;
     it.hslot = local - rank * n_heads;
     it.qt = nt - 1 - rank;
     return it;
+}
+
+__device__ __forceinline__ LseItem decode_lse_item_at(int item, int b, const int32_t* base,
+                                                      const int32_t* cu, int tile, int n_heads) {
+    return decode_lse_item_at(item, b, b, base, cu, tile, n_heads);
 }
 
 __device__ __forceinline__ LseItem decode_lse_item(int item, const int32_t* base, int B,

@@ -798,8 +798,8 @@ static bool lse_head_pairs(const ImpHeads& hs) {
 }
 
 PlanReq lse_plan_tc(const ImpHeads& hs, int32_t* base, PlanInfo* info) {
-    return lse_head_pairs(hs) ? PlanReq{kTile, 1, hs.n_heads / 2, 1, base, info}
-                              : PlanReq{kPair, 1, hs.n_heads, 1, base, info};
+    return lse_head_pairs(hs) ? PlanReq{kTile, 1, hs.n_heads / 2, 1, base, info, 0}
+                              : PlanReq{kPair, 1, hs.n_heads, 1, base, info, 0};
 }
 
 estp_status launch_lse_tc(estp_ctx* ctx, const void* Q, const void* K, int Hq, int Hkv, int d,

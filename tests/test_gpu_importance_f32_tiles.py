@@ -1,6 +1,6 @@
 """fp32 row normalisers and column sums at the edges of their tiles, in each split of the work
-(64 or 128 fixed rows, chunks of 1 to 8 query tiles, items per head or per KV group), against
-the oracle (GPU)."""
+(64 or 128 fixed rows, chunks of 1 to 8 query tiles, items per head or per KV group, prompts in
+batch order or in order of length), against the oracle (GPU)."""
 import math
 
 import numpy as np
@@ -18,6 +18,8 @@ CASES = {
     "one": ([1], 1, 1, 64),
     "edges64": ([63, 64, 65, 0, 127], 2, 1, 128),
     "edges128": ([128, 129, 191, 192, 193], 4, 2, 64),
+    # more items than blocks: prompts in order of length
+    "sorted": ([0, 700, 1, 0, 640, 300, 640, 900], 8, 8, 64),
     # column sums with 128 rows and one query tile per item
     "edges256": ([255, 256, 257, 320, 385, 448, 511, 640], 8, 2, 64),
     # 128 rows for both, items per KV group, chunks of 8 query tiles

@@ -816,7 +816,7 @@ def time_head_loss(st, dev):
     ms = _time_calls(lambda: st.ctx.head_loss(st.pooled, st.head, targets, 0.5),
                      st.ctx.sync_status, min_warm_s=0.05, want_s=0.05)
     nbytes = 4 * (2 * K * D + 2 * B * D + K * D + K + B * D + B * K)
-    out = {"ms": ms, "B": B, "D": D, "K": K, "launches": 2, "bytes": nbytes,
+    out = {"ms": ms, "B": B, "D": D, "K": K, "launches": 3, "bytes": nbytes,
            "achieved_gbs": nbytes / (ms / 1e3) / 1e9, "bound": "launch"}
     # the MLP predictor (one ReLU layer of F = 1024 units), its loss and all gradients
     F = 1024
@@ -828,7 +828,7 @@ def time_head_loss(st, dev):
                      st.ctx.sync_status, min_warm_s=0.05, want_s=0.05)
     # W1 read by the hidden layer and by both of its gradients, dL/dW1 written
     mbytes = 4 * (3 * F * D + F * D + 2 * K * F + 4 * B * D + 4 * B * F)
-    out["mlp"] = {"ms": ms, "F": F, "launches": 5, "bytes": mbytes,
+    out["mlp"] = {"ms": ms, "F": F, "launches": 6, "bytes": mbytes,
                   "achieved_gbs": mbytes / (ms / 1e3) / 1e9, "bound": "launch / L2"}
     return out
 

@@ -64,6 +64,7 @@ void launch_plans(estp_ctx* ctx, const int32_t* cu, int B, int64_t sumT, int max
 }
 
 // Workspace bytes of a plan, and its two parts.
+static_assert(sizeof(PlanInfo) <= 256, "the info part of a plan");
 inline size_t plan_bytes(int B) { return align_up(sizeof(int32_t) * (size_t)(B + 1), 256) + 256; }
 inline int32_t* plan_base(char* ws) { return reinterpret_cast<int32_t*>(ws); }
 inline PlanInfo* plan_info(char* ws, int B) {

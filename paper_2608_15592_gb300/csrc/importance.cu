@@ -89,7 +89,8 @@ static __device__ void plan_body(const int32_t* cu, int B, int64_t sumT, int max
 }
 
 __global__ void __launch_bounds__(1024) attn_plan_kernel(const int32_t* cu, int B, int64_t sumT,
-                                                         int max_seqlen, const PlanSet plans,
+                                                         int max_seqlen,
+                                                         const __grid_constant__ PlanSet plans,
                                                          int* status) {
     // the tensor-core kernel that consumes the plan may launch now and run its prologue;
     // it waits for this grid before its first read of the plan

@@ -24,6 +24,7 @@
 // Every mbarrier wait is bounded (a test may lower the limit of the abortable waits
 // through estp_set_wait_limit); on expiry the CTA records ESTP_ERR_TIMEOUT in the status
 // word, drains its own copies and MMAs and frees its TMEM.
+#include "split_rules.cuh"
 #include "tcgen05.cuh"
 
 namespace estp {
@@ -31,7 +32,7 @@ namespace {
 
 constexpr int kM = 128;                       // tokens per tile (TMEM lanes)
 constexpr int kN = 256;                       // vocabulary entries per tile (MMA N)
-constexpr int kUnit = 32;                     // granularity of a split and of its last tile
+constexpr int kUnit = 32;                     // granularity of a tile that is not full
 constexpr int kKc = 64;                       // hidden-size chunk per stage (one swizzle atom)
 constexpr int kStages = 4;
 constexpr int kABytes = kM * kKc * 2;         // 16 KB
@@ -54,6 +55,7 @@ struct LmArgs {
     int nk;            // hidden-size chunks (D / 64)
     int n_unit;        // vocabulary units of kUnit entries
     int S;             // vocabulary splits
+    int gran;          // units a split is cut in (1, or a whole tile)
     int a_bytes;       // bytes of a stage's A box: 128 rows, or the rows of a single smaller block
     int64_t n_items;   // row blocks x splits
     float* part;       // [3][S][n_rows]: m, s, t (log2 units)
@@ -61,14 +63,15 @@ struct LmArgs {
     long long wait_cycles;  // limit of the abortable waits (kWaitCycles unless a test lowers it)
 };
 
-// Vocabulary units [u0, u1) of split sp.  Splits are cut in units and not in whole tiles, so
-// that every CTA gets the same share of W whatever V is (V = 128256 is 501 tiles, 3.3 for each of
-// 152 SMs); a split's last tile loads and multiplies only the units it has.
+// Vocabulary units [u0, u1) of split sp: lm_split says when splits end inside a tile.  Such a last
+// tile loads and multiplies only the units it has.
 __device__ __forceinline__ void split_range(const LmArgs& a, int sp, int& u0, int& u1) {
-    u0 = (int)((int64_t)sp * a.n_unit / a.S);
-    u1 = (int)((int64_t)(sp + 1) * a.n_unit / a.S);
+    const int64_t n = (a.n_unit + a.gran - 1) / a.gran;
+    u0 = (int)(sp * n / a.S) * a.gran;
+    u1 = min(a.n_unit, (int)((sp + 1) * n / a.S) * a.gran);
 }
 constexpr int kTileUnits = kN / kUnit;
+static_assert(kTileUnits == kLmTileUnits, "units of a tile");
 
 // D (TMEM) = A B^T (+ D when acc != 0) with N = n columns.
 __device__ __forceinline__ void mma_n(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t n, uint32_t acc) {
@@ -301,9 +304,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // Per token: the splits' (m, s, t) combined, H in nats.  A block takes 32 tokens; its warp y the
 // splits y, y + Y, .. of each in order, and the Y results are combined in warp order (a fixed
-// order, whatever the launch).  A small batch has as many splits as vocabulary tiles (594 for 37
-// tokens of a 152064-entry vocabulary), which one thread a token read one after another: 198 us there
-// (the call 342 us, against 176 now).  Launched as a programmatic dependent of lm_head_kernel.
+// order, whatever the launch).  A single row block has a split per SM (152).  One thread a token,
+// which read its splits one after another, took 198 us with the 594 whole-tile splits that 37
+// tokens of a 152064-entry vocabulary had then (the call 342 us, against 176 now).  Launched as a
+// programmatic dependent of lm_head_kernel.
 constexpr int kMergeWarps = 32;
 __device__ __forceinline__ void merge_split(float& M, float& S, float& T, float m, float s, float t) {
     const float mm = fmaxf(M, m);
@@ -390,30 +394,15 @@ estp_status launch_lm_head_entropy(estp_ctx* ctx, const void* hidden, int64_t ld
     a.nk = (int)(D / kKc);
     a.n_unit = (int)((V + kUnit - 1) / kUnit);
     const int64_t n_rb = (n_rows + kM - 1) / kM;
-    // splits: the fewest whose items fill the last wave of the persistent grid to 97 % (else
-    // the best fill up to four times as many).  Fewer splits keep more row blocks in flight at
-    // once, so that each W tile read from DRAM serves more of them.  (Cut in units of 32 entries the
-    // splits are equal, so one item an SM is enough: at least four, cut in whole tiles, took 3026 us
-    // for 4103 x 4096 x 128256 against 2731, 604 against 512 for 1291 x 3776 x 68767.)
-    // At least as many splits that the row blocks in flight at once (G / S of them, 256 D
-    // bytes each) fit in ~48 MB of L2 beside the W tiles streaming through.
+    // vocabulary splits: at least as many that the row blocks in flight at once (G / S of them,
+    // 256 D bytes each) fit in ~48 MB of L2 beside the W tiles streaming through
     const int64_t G = ctx->num_sms;
     const int64_t l2_budget = 48ll << 20, rb_bytes = (int64_t)kM * D * 2;
     const int64_t s_l2 = (G * rb_bytes + l2_budget - 1) / l2_budget;
-    int64_t s_lo = G / n_rb > 0 ? G / n_rb : 1;
-    if (s_lo < s_l2) s_lo = s_l2;
-    int64_t S = s_lo < a.n_unit ? s_lo : a.n_unit;  // small problems: one unit per split
-    double best = -1.0;
-    for (int64_t c = s_lo; c <= a.n_unit && c <= 4 * s_lo; ++c) {
-        const int64_t items = n_rb * c, waves = (items + G - 1) / G;
-        const double fill = (double)items / (double)(waves * G);
-        if (fill > best + 1e-9) {
-            best = fill;
-            S = c;
-        }
-        if (fill >= 0.97) break;
-    }
+    const LmSplit cut = lm_split(n_rb, a.n_unit, s_l2, G);
+    const int64_t S = cut.S;
     a.S = (int)S;
+    a.gran = cut.gran;
     a.a_bytes = a_rows * kKc * 2;
     a.n_items = n_rb * S;
     s = ws_reserve(ctx, sizeof(float) * 3 * (size_t)S * (size_t)n_rows);

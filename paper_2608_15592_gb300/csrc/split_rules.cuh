@@ -1,0 +1,57 @@
+// How the launchers cut their work: host rules on sizes alone, in plain C++ (no CUDA), so that they
+// can be checked without a device.
+#pragma once
+#include <stdint.h>
+
+namespace estp {
+
+inline int64_t div_up(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// ---------------------------------------------------------------- entropy from hidden states
+// n_rb row blocks x S vocabulary splits are dealt round-robin to one CTA an SM.  A split is cut in
+// cuts of `gran` units (32 entries) and worked off in tiles of kLmTileUnits; a tile that is not full
+// takes as long as a full one or longer (its A box is loaded all the same, and its W box unit by
+// unit), so splits are whole tiles.  Only where W is the bound (a single row block: every CTA streams
+// its own share) or where whole tiles do not give every SM an item are they cut in units, which are
+// equal within one.  Whole tiles against units, the same S: 20000 rows, D 4096, V 8000 850 and 920
+// us; 3000 rows there 140 and 142; 256 rows, V 32000 72.2 and 80.3; one row, V 128256 180.7 and 176.6.
+constexpr int kLmTileUnits = 8;
+
+struct LmSplit {
+    int64_t S;
+    int gran;
+};
+
+// S minimises, for the SM with the most items, its cuts plus what each item costs beside them, over
+// up to 16 items an SM (or four times the fewest).  An item costs its share of one more pass of W
+// through L2: with S forced it came to a 40th to a 100th of the vocabulary.  Of the splits with the
+// same number of items an SM the largest is the best, so one per number is looked at.  Measured
+// sustained over 37 sizes (129 to 21663 rows, D 896 to 4096, V 5000 to 152064) with 8 to 10 S each:
+// the rule's S is within 1.8 % of the best one.  A rule that took the first S whose last round is
+// 97 % full, of at most four times the fewest, left SMs idle or took rounds that cost more than
+// they filled: 14848 rows, D 896, V 128256 2370 us for S = 1 against 2154 for 5; 20000 rows, D 4096,
+// V 8000 996 against 902; 5888 rows, D 4096, V 128256 4004 for S = 13 against 3851 for 6.
+constexpr int kLmPassShare = 64;
+
+// s_min: at least as many splits as keep the row blocks in flight in L2.
+inline LmSplit lm_split(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t num_sms) {
+    const int64_t n_tile = div_up(n_unit, kLmTileUnits);
+    const bool whole = n_rb > 1 && n_rb * n_tile >= num_sms;
+    const int64_t n = whole ? n_tile : n_unit;
+    LmSplit best{n < s_min ? n : s_min, whole ? kLmTileUnits : 1};
+    const int64_t w0 = div_up(n_rb * best.S, num_sms);  // items of the busiest SM
+    const int64_t w1 = 4 * w0 > 16 ? 4 * w0 : 16;
+    int64_t best_cost = INT64_MAX;
+    for (int64_t w = w0; w <= w1; ++w) {
+        const int64_t S = w * num_sms / n_rb < n ? w * num_sms / n_rb : n;
+        const int64_t cost = div_up(n_rb * S, num_sms) * (kLmPassShare * div_up(n, S) + n);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best.S = S;
+        }
+        if (S == n) break;
+    }
+    return best;
+}
+
+}  // namespace estp

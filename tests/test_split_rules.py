@@ -1,0 +1,88 @@
+"""The host rules that cut the launchers' work (csrc/split_rules.cuh), on the CPU: compiled with the
+host compiler and compared, over the whole range of sizes, with what a device would do with them."""
+import ctypes
+import os
+import random
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SMS = 152
+
+SRC = """
+#include "split_rules.cuh"
+using namespace estp;
+extern "C" void lm(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t sms, int64_t* S, int* gran) {
+    const LmSplit r = lm_split(n_rb, n_unit, s_min, sms);
+    *S = r.S;
+    *gran = r.gran;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    d = tmp_path_factory.mktemp("rules")
+    (d / "rules.cpp").write_text(SRC)
+    lib = str(d / "rules.so")
+    subprocess.run([cxx, "-std=c++17", "-Wall", "-Wextra", "-Werror", "-O1", "-shared", "-fPIC", "-I",
+                    os.path.join(ROOT, "paper_2608_15592_gb300", "csrc"), str(d / "rules.cpp"), "-o", lib], check=True)
+    return ctypes.CDLL(lib)
+
+
+def _up(a, b):
+    return -(-a // b)
+
+
+# ------------------------------------------------------------ entropy from hidden states
+def _lm(rules, n_rb, n_unit, s_min):
+    S, gran = ctypes.c_int64(), ctypes.c_int()
+    i = ctypes.c_int64
+    rules.lm(i(n_rb), i(n_unit), i(s_min), i(SMS), ctypes.byref(S), ctypes.byref(gran))
+    return S.value, gran.value
+
+
+def _lm_busiest(n_rb, n_unit, S, gran):
+    """Tiles of the busiest SM and its items: items round-robin, split fastest, a tile that is not
+    full counted whole."""
+    n = _up(n_unit, gran)
+    cut = [min(n_unit, sp * n // S * gran) for sp in range(S + 1)]
+    assert cut[0] == 0 and cut[-1] == n_unit and all(b > a for a, b in zip(cut, cut[1:]))
+    tiles = [_up(b - a, 8) for a, b in zip(cut, cut[1:])]
+    load = [0] * SMS
+    for item in range(n_rb * S):
+        load[item % SMS] += tiles[item % S]
+    return max(load), _up(n_rb * S, SMS)
+
+
+def _lm_cost(n_rb, n_unit, S, gran):
+    tiles, items = _lm_busiest(n_rb, n_unit, S, gran)
+    return tiles + items * _up(n_unit, 8) / 64  # an item costs its share of one more pass of W
+
+
+@pytest.mark.parametrize("V", [8000, 32000, 50257, 128256, 152064])
+def test_lm_split_leaves_no_sm_idle(rules, V):
+    n_unit = _up(V, 32)
+    rng = random.Random(V)
+    for n_rb in {1, 2, 3, 5, 36, 46, 66, 71, 77, 116, 130, 143, 170, *(rng.randint(2, 470) for _ in range(40))}:
+        for s_min in (1, 2, 4):  # D up to 1280, 2048, 4096
+            S, gran = _lm(rules, n_rb, n_unit, s_min)
+            assert s_min <= S <= _up(n_unit, gran)
+            got = _lm_cost(n_rb, n_unit, S, gran)
+            # every number of splits the kernel could take, up to sixteen items an SM
+            top = max(4 * s_min, _up(16 * SMS, n_rb))
+            best = min(_lm_cost(n_rb, n_unit, s, 8) for s in range(s_min, min(top, _up(n_unit, 8)) + 1))
+            # (the rule takes every item for the largest, a real SM has some smaller ones)
+            assert got <= 1.06 * best + 1, (n_rb, s_min, S, gran, got, best)
+
+
+@pytest.mark.parametrize("n_rb,n_unit,s_min", [(1, 1, 1), (1, 2, 4), (3, 4, 13), (470, 1, 1), (5000, 4008, 4)])
+def test_lm_split_small(rules, n_rb, n_unit, s_min):
+    S, gran = _lm(rules, n_rb, n_unit, s_min)
+    assert 1 <= S <= _up(n_unit, gran)
+    _lm_busiest(n_rb, n_unit, S, gran)

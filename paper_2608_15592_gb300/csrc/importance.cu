@@ -380,12 +380,6 @@ struct F32Split {
     bool per_head;
 };
 
-// Tiles of a prompt of mean length: the lengths themselves stay on the device.
-int64_t mean_tiles(int B, int64_t sumT, int rows) {
-    const int64_t t = B > 0 ? (sumT + B - 1) / B : 0;
-    return (t + rows - 1) / rows;
-}
-
 int f32_rows(int B, int64_t sumT, int n_heads, int num_sms) {
     return (int64_t)B * n_heads * mean_tiles(B, sumT, 128) >= (int64_t)kFLseItemsPerSm * num_sms ? 128 : 64;
 }

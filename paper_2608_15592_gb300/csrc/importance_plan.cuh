@@ -13,13 +13,9 @@
 // largest items of a prompt first.
 #pragma once
 #include "estp_internal.cuh"
+#include "split_rules.cuh"
 
 namespace estp {
-
-__host__ __device__ __forceinline__ int64_t items_f(int64_t n, int qc) {
-    const int64_t a = n / qc, r = n % qc;
-    return (int64_t)qc * a * (a + 1) / 2 + r * (a + 1);
-}
 
 constexpr int kMaxSorted = 64;  // prompts of a plan in order of length
 
@@ -147,11 +143,6 @@ __device__ __forceinline__ LseItem decode_lse_item_at(int item, int b, const int
 __device__ __forceinline__ LseItem decode_lse_item(int item, const int32_t* base, int B,
                                                    const int32_t* cu, int tile, int n_heads) {
     return decode_lse_item_at(item, upper_slot(base, B, item), base, cu, tile, n_heads);
-}
-
-// Number of chunks of key tile kt of a prompt with nt tiles.
-__host__ __device__ __forceinline__ int chunks_of(int nt, int kt, int qc) {
-    return (nt - kt + qc - 1) / qc;
 }
 
 }  // namespace estp

@@ -53,13 +53,6 @@ namespace {
 
 constexpr int kTile = 128;             // rows of a fixed or streamed tile
 constexpr int kPair = 2 * kTile;       // rows of the fixed pair (the plan's tile)
-// Pairs of query tiles per column-sum item: the largest of kQcChoices that still gives the
-// persistent grid about kItemsPerSm items per SM (tc_qc).  Longer items cost fewer item
-// hand-offs; too few items leave SMs idle at the end of a launch.  One pair per item where two
-// would not give every SM an item: one prompt of 1024 tokens 34.4 -> 24.8 us, of 2048 35.3 ->
-// 26.6, four of 300 23.2 -> 21.0; from there on it costs up to 8 %.
-constexpr int kQcChoices[4] = {16, 8, 4, 2};
-constexpr int kItemsPerSm = 16;
 constexpr int kEpiWarp0 = 2;           // warps 2..17
 constexpr int kEpiWarps = 16;          // 8 per fixed tile
 // MMA issuers: warp 1 for fixed tile A, warp 18 for tile B, so that one issuer's barrier
@@ -780,14 +773,7 @@ estp_status launch_tc(estp_ctx* ctx, const CUtensorMap& fixm, const CUtensorMap&
 
 bool tc_supported(estp_dtype dtype, int d) { return dtype == ESTP_BF16 && (d == 64 || d == 128); }
 int tc_tile() { return kPair; }
-int tc_qc(int B, int64_t sumT, int n_groups, int num_sms) {
-    // the prompts' lengths stay on the device: estimate the item count from the mean length
-    const int64_t t_mean = B > 0 ? (sumT + B - 1) / B : 0;
-    const int64_t nt = (t_mean + kPair - 1) / kPair;
-    for (int qc : kQcChoices)
-        if ((int64_t)B * n_groups * items_f(nt, qc) >= (int64_t)kItemsPerSm * num_sms) return qc;
-    return (int64_t)B * n_groups * items_f(nt, kQcChoices[3]) < num_sms ? 1 : kQcChoices[3];
-}
+int tc_qc(int B, int64_t sumT, int n_groups, int num_sms) { return imp_pairs(B, sumT, n_groups, kPair, num_sms); }
 
 // LSE items: (prompt, query tile, pair of heads of one KV group) when every group holds an
 // even number of the selected heads, else (prompt, pair of query tiles, head)

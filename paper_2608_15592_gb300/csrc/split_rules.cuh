@@ -1,11 +1,47 @@
-// How the launchers cut their work: host rules on sizes alone, in plain C++ (no CUDA), so that they
-// can be checked without a device.
+// How the launchers cut their work: host rules on sizes alone, in plain C++, so that they can be
+// checked without a device.
 #pragma once
 #include <stdint.h>
 
+#ifdef __CUDACC__
+#define ESTP_RULE __host__ __device__ __forceinline__
+#else
+#define ESTP_RULE inline
+#endif
+
 namespace estp {
 
-inline int64_t div_up(int64_t a, int64_t b) { return (a + b - 1) / b; }
+ESTP_RULE int64_t div_up(int64_t a, int64_t b) { return (a + b - 1) / b; }
+
+// --------------------------------------------------------------- attention importance items
+// Items of one group of a prompt of n tiles, cut into chunks of qc query tiles (importance_plan.cuh).
+ESTP_RULE int64_t items_f(int64_t n, int qc) {
+    const int64_t a = n / qc, r = n % qc;
+    return (int64_t)qc * a * (a + 1) / 2 + r * (a + 1);
+}
+
+// Number of chunks of key tile kt of a prompt with nt tiles.
+ESTP_RULE int chunks_of(int nt, int kt, int qc) { return (nt - kt + qc - 1) / qc; }
+
+// Tiles of a prompt of mean length: the lengths themselves stay on the device.
+inline int64_t mean_tiles(int B, int64_t sumT, int rows) {
+    return div_up(B > 0 ? div_up(sumT, B) : 0, rows);
+}
+
+// Pairs of query tiles per column-sum item of bf16 inputs (tiles are pairs of `pair` rows): the
+// largest of 16, 8, 4 and 2 that still gives about kImpItemsPerSm items an SM.  Longer items cost
+// fewer item hand-offs; too few items leave SMs idle at the end of a launch.  One pair per item where
+// every SM then has at most one: one prompt of 1000 tokens, 28/4 heads, 33.0 -> 22.8 us, of 2000
+// 34.8 -> 25.1, three of 1000 35.0 -> 24.8.  Where one pair makes more items than SMs, two are as
+// good or better (fewer partials to add): one prompt of 1000, 16/16 heads, 18.5 for one pair and
+// 16.6 for two, of 2300, 28/4 heads, 37.0 and 35.1, of 1500, 32/8 heads, 28.3 and 26.8.
+constexpr int kImpItemsPerSm = 16;
+inline int imp_pairs(int B, int64_t sumT, int n_groups, int pair, int num_sms) {
+    const int64_t lists = (int64_t)B * n_groups, nt = mean_tiles(B, sumT, pair);
+    for (int qc = 16; qc >= 2; qc /= 2)
+        if (lists * items_f(nt, qc) >= (int64_t)kImpItemsPerSm * num_sms) return qc;
+    return lists * items_f(nt, 1) <= num_sms ? 1 : 2;
+}
 
 // ---------------------------------------------------------------- entropy from hidden states
 // n_rb row blocks x S vocabulary splits are dealt round-robin to one CTA an SM.  A split is cut in

@@ -19,6 +19,7 @@ extern "C" void lm(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t sms, int
     *S = r.S;
     *gran = r.gran;
 }
+extern "C" int pairs(int B, int64_t sumT, int n_groups, int sms) { return imp_pairs(B, sumT, n_groups, 256, sms); }
 """
 
 
@@ -86,3 +87,22 @@ def test_lm_split_small(rules, n_rb, n_unit, s_min):
     S, gran = _lm(rules, n_rb, n_unit, s_min)
     assert 1 <= S <= _up(n_unit, gran)
     _lm_busiest(n_rb, n_unit, S, gran)
+
+
+# ------------------------------------------------------------------- column sums (bf16)
+def _items(n, qc):
+    return sum(_up(m, qc) for m in range(1, n + 1))
+
+
+@pytest.mark.parametrize("n_groups", [1, 2, 4, 8, 16])
+def test_column_sum_items_of_one_pair_fit_the_sms(rules, n_groups):
+    for B in (1, 2, 3, 4, 7, 8, 16, 40, 160):
+        for T in (1, 100, 256, 257, 300, 700, 1000, 1500, 2300, 4000, 9000, 40000):
+            nt = _up(T, 256)
+            qc = rules.pairs(B, ctypes.c_int64(B * T), n_groups, SMS)
+            items = B * n_groups * _items(nt, qc)
+            if qc == 1:
+                assert items <= SMS, (B, T)
+            else:  # two pairs wherever one pair would not fit and longer items would leave SMs idle
+                assert B * n_groups * _items(nt, 1) > SMS, (B, T)
+                assert qc == 2 or items >= 16 * SMS, (B, T)

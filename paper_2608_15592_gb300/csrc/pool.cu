@@ -19,9 +19,8 @@
 // counter) adds the partials in column-block order and reduces the head.  The merge
 // and the head run after the stream, when their short dependent reads meet an idle
 // memory system.  No floating-point atomics: every sum runs in a fixed order.
-#include <cmath>
-
 #include "estp_internal.cuh"
+#include "split_rules.cuh"
 
 namespace estp {
 namespace {
@@ -31,12 +30,6 @@ constexpr int kMaxThreads = 512;  // stream CTA: 16-byte column units of one sli
 constexpr int kBatch = 4;         // rows per load batch; two batches in flight per thread
 constexpr int kFinThreads = 512;  // finish CTA: 2 columns per thread
 constexpr int kFinCols = 2 * kFinThreads;
-// G ranges of a batch of B prompts take about bytes / (G x 54 GB/s) to stream below the memory's
-// rate (one CTA's loads in flight) and G / B slots a prompt, 75 ns each, to merge: the sum is
-// least at G^2 = bytes B / kRangeBytes.  One wave against this rule, pooling and head: one prompt
-// of 128 x 1024 fp32 15.4 -> 10.4 us, 300 x 4096 bf16 29.8 -> 13.4, 2048 x 3584 29.3 -> 18.3,
-// 8192 x 4096 34.5 -> 26.0; from 16 prompts of 1300 on the wave is full either way.
-constexpr double kRangeBytes = 4000.0;
 constexpr int kMaxSlots = 1024;   // slot factors staged per pass of the finish kernel
 
 struct StreamArgs {
@@ -399,13 +392,9 @@ estp_status launch_pool(estp_ctx* ctx, const void* hidden, estp_dtype dtype, int
     int occ = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, threads, 0);
     if (e != cudaSuccess) return cuda_fail(e, "pool occupancy");
-    // one wave: G token ranges x n_slices column slices, every range with >= 1 token, or fewer
-    // ranges for a small batch (kRangeBytes)
-    int64_t G = (int64_t)ctx->num_sms * (occ > 0 ? occ : 1) / n_slices;
-    const double few = std::sqrt((double)sumT * (double)D * esize(dtype) * B / kRangeBytes);
-    if ((double)G > few) G = (int64_t)few;
-    if (G < 1) G = 1;
-    if (sumT > 0 && G > sumT) G = sumT;
+    // one wave of G token ranges x n_slices column slices, or fewer ranges for a small batch
+    const int64_t full = (int64_t)ctx->num_sms * (occ > 0 ? occ : 1) / n_slices;
+    const int64_t G = pool_ranges(sumT, D * esize(dtype), B, full > 1 ? full : 1, n_slices, ctx->num_sms);
     a.G = (int)G;
     a.H = H;
     a.S = S;

@@ -1,6 +1,7 @@
 // How the launchers cut their work: host rules on sizes alone, in plain C++, so that they can be
 // checked without a device.
 #pragma once
+#include <math.h>
 #include <stdint.h>
 
 #ifdef __CUDACC__
@@ -88,6 +89,32 @@ inline LmSplit lm_split(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t num
         if (S == n) break;
     }
     return best;
+}
+
+// ------------------------------------------------------------------------------------ pooling
+// Token ranges of the pooling stream, each streamed by one CTA per column slice; `full` ranges
+// (full x n_slices CTAs) are one wave.  G ranges of a batch of B prompts take about
+// bytes / (G x 54 GB/s) to stream below the memory's rate (one CTA's loads in flight) and G / B slots
+// a prompt, 75 ns each, to merge: the sum is least at G^2 = bytes B / kPoolRangeBytes.  One wave
+// against this, pooling and head: one prompt of 128 x 1024 fp32 15.4 -> 10.4 us, 300 x 4096 bf16
+// 29.8 -> 13.4, 2048 x 3584 29.3 -> 18.3, 8192 x 4096 34.5 -> 26.0.
+// CTAs of which an SM holds two (rows of 7 KB and more) are one on each SM or a wave: between the two
+// the SMs with two set the pace.  16 prompts of 16 to 100 tokens x 4096 bf16 24.7 us with 177 CTAs,
+// 20.7 with 152, 22.9 with 304; 8 x 700 x 4096 26.9 with 303, 22.6 with 152, 24.7 with 304.  (Smaller
+// CTAs are limited by their own loads: 16 x 256..2048 x 512 bf16 20.7 us with 281, 25.5 with 152.)  A
+// wave that would be five sixths full is filled: 64 x 512 x 512 fp32 18.9 us with 1036, 18.6 with 1216.
+constexpr double kPoolRangeBytes = 4000.0;
+inline int64_t pool_ranges(int64_t sumT, int64_t row_bytes, int B, int64_t full, int n_slices, int num_sms) {
+    int64_t G = full;
+    const double few = sqrt((double)sumT * (double)row_bytes * B / kPoolRangeBytes);
+    if ((double)G > few) {
+        G = (int64_t)few;
+        const int64_t two = 2 * (int64_t)num_sms;
+        if (full * n_slices <= two && G * n_slices > num_sms && G * n_slices < two) G = num_sms / n_slices;
+        else if (6 * G >= 5 * full) G = full;
+    }
+    if (G > sumT) G = sumT;
+    return G > 1 ? G : 1;  // every range holds >= 1 token
 }
 
 }  // namespace estp

@@ -19,6 +19,9 @@ extern "C" void lm(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t sms, int
     *S = r.S;
     *gran = r.gran;
 }
+extern "C" int64_t ranges(int64_t sumT, int64_t row_bytes, int B, int64_t full, int n_slices, int sms) {
+    return pool_ranges(sumT, row_bytes, B, full, n_slices, sms);
+}
 extern "C" int pairs(int B, int64_t sumT, int n_groups, int sms) { return imp_pairs(B, sumT, n_groups, 256, sms); }
 """
 
@@ -106,3 +109,25 @@ def test_column_sum_items_of_one_pair_fit_the_sms(rules, n_groups):
             else:  # two pairs wherever one pair would not fit and longer items would leave SMs idle
                 assert B * n_groups * _items(nt, 1) > SMS, (B, T)
                 assert qc == 2 or items >= 16 * SMS, (B, T)
+
+
+# ---------------------------------------------------------------------------- pooling
+@pytest.mark.parametrize("row_bytes,ctas_per_sm,n_slices", [(2048, 8, 1), (4096, 4, 1), (7168, 2, 1), (8192, 2, 1),
+                                                            (16384, 2, 2), (65536, 2, 8)])
+def test_pool_ranges_balance_the_sms(rules, row_bytes, ctas_per_sm, n_slices):
+    i = ctypes.c_int64
+    rules.ranges.restype = i
+    full = SMS * ctas_per_sm // n_slices
+    for B in (1, 2, 8, 16, 64, 256):
+        for T in (1, 2, 16, 58, 100, 300, 700, 2048, 8192):
+            sumT = B * T
+            G = rules.ranges(i(sumT), i(row_bytes), B, i(full), n_slices, SMS)
+            assert 1 <= G <= min(full, sumT), (B, T)
+            ctas = G * n_slices
+            if sumT >= full and G < full:
+                # no SM with two large CTAs among SMs with one, and no wave that is nearly full
+                assert ctas <= SMS or ctas >= 2 * SMS or ctas_per_sm > 2, (B, T, G)
+                assert ctas <= SMS or 6 * G < 5 * full, (B, T, G)
+                # enough ranges in flight for the bytes, few enough slots to merge
+                want = (sumT * row_bytes * B / 4000) ** 0.5
+                assert 0.45 * want <= G <= want, (B, T, G)

@@ -14,8 +14,8 @@
 //   layer_grad_kernel: tiles of dL/dW = sum_b dz_b x_b^T and of dL/dx_b = W^T dz_b, with
 //     dL/dbias = sum_b dz_b along the first column of tiles, and one block for the loss.
 // The MLP adds wide_gemm_kernel, u = max(W1 h + b1, 0) and dL/dh = W1^T g, cut along its
-// contraction over a cluster whose CTAs add their tiles through distributed shared memory,
-// and outer_kernel, dL/dW1 = g^T h with dL/db1; g = dL/du where u > 0 (the ReLU's
+// contraction over a cluster whose CTAs add their tiles through distributed shared memory
+// (hidden_rows_kernel forms u for at most 8 prompts), and outer_kernel, dL/dW1 = g^T h with dL/db1; g = dL/du where u > 0 (the ReLU's
 // derivative), formed by layer_grad_kernel.  Every sum runs in a fixed order.
 //
 // Measured, 256 prompts, D = 4096, K = 32 (GB300, device times with cold caches):
@@ -325,6 +325,44 @@ __global__ void __launch_bounds__(256, 2) outer_kernel(GemmSide g, GemmSide h, i
     }
 }
 
+// u[b, f] = max(sum_x W1[f, x] h[b, x] + b1[f], 0) for a batch of at most NB prompts: one warp a
+// hidden unit, lanes along D four columns at a time, then a fixed butterfly.  With so few prompts
+// reading W1 is the bound, and a tile of wide_gemm_kernel has only a slice of it in flight (one
+// prompt, 4096 x 1024: 31 us cold, which is 0.5 TB/s).  Prediction through the MLP, F 1024, with that
+// kernel and with this one: 1 prompt, D 4096, 32 bins 35.7 and 18.5 us; 4 prompts, D 8192, 128 bins
+// 65.8 and 35.0; 8 prompts, D 4096, 32 bins 37.0 and 24.7, with cold caches 39.9 and 37.9.  For 16
+// prompts the tiles are as good, with cold caches better (35.8 against 39.9).
+constexpr int kRowBatch = 8;
+template <int NB>
+__global__ void __launch_bounds__(128) hidden_rows_kernel(GemmSide h, GemmSide w, int64_t D,
+                                                          const float* __restrict__ bias, float* __restrict__ u) {
+    chain_launches();
+    const int lane = threadIdx.x & 31;
+    const int64_t f = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (f >= w.rows) return;
+    float2 acc[NB][2];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+    for (int64_t x = 4 * lane; x < D; x += 128) {
+        // every load of the pass first (prompts past the batch read as zero), then the FMAs
+        const float4 wv = LogitTile::fetch<true>(w, f, x, D);
+        float4 hv[NB];
+#pragma unroll
+        for (int j = 0; j < NB; ++j) hv[j] = LogitTile::fetch<true>(h, j, x, D);
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            acc[j][0] = __ffma2_rn(make_float2(wv.x, wv.y), make_float2(hv[j].x, hv[j].y), acc[j][0]);
+            acc[j][1] = __ffma2_rn(make_float2(wv.z, wv.w), make_float2(hv[j].z, hv[j].w), acc[j][1]);
+        }
+    }
+    const float b = bias ? bias[f] : 0.f;
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+        const float v = warp_sum((acc[j][0].x + acc[j][0].y) + (acc[j][1].x + acc[j][1].y)) + b;
+        if (lane == 0 && j < h.rows) u[j * w.rows + f] = v > 0.f ? v : 0.f;
+    }
+}
+
 // A matrix with `rows` rows of `n` contiguous floats: as an operand whose side is the rows
 // (k along a row) or whose side is the columns (k over the rows).
 GemmSide side_rows(const float* p, int64_t rows, int64_t n) {
@@ -421,6 +459,16 @@ cudaError_t wide_gemm(estp_ctx* ctx, const GemmSide& A, const GemmSide& Bm, int6
                    : go(wide_gemm_kernel<1, 64, kAlongB, kRelu>);
 }
 
+// The hidden layer u = max(W1 h + b1, 0), the first launch of its call.
+cudaError_t hidden_layer(estp_ctx* ctx, const float* pooled, int B, int64_t D, const estp_mlp_head& head, float* u,
+                         cudaStream_t st) {
+    const GemmSide h = side_rows(pooled, B, D), w = side_rows(head.W1, head.F, D);
+    if (B > kRowBatch) return wide_gemm<true, true>(ctx, h, w, D, head.b1, u, false, st);
+    auto go = [&](auto kern) { return launch(kern, dim3((unsigned)ceil_div(head.F, 4)), 128, st, false, 1, h, w, D, head.b1, u); };
+    return B > 4 ? go(hidden_rows_kernel<8>) : B > 2 ? go(hidden_rows_kernel<4>)
+         : B > 1 ? go(hidden_rows_kernel<2>) : go(hidden_rows_kernel<1>);
+}
+
 }  // namespace
 
 estp_status launch_head_loss(estp_ctx* ctx, const float* pooled, int B, int64_t D,
@@ -457,7 +505,7 @@ estp_status launch_mlp_head_predict(estp_ctx* ctx, const float* pooled, int B, i
     if (s != ESTP_OK) return s;
     char* ws = static_cast<char*>(ctx->ws);
     float* u = reinterpret_cast<float*>(ws);
-    cudaError_t e = wide_gemm<true, true>(ctx, side_rows(pooled, B, D), side_rows(head.W1, F, D), D, head.b1, u, false, st);
+    cudaError_t e = hidden_layer(ctx, pooled, B, D, head, u, st);
     if (e != cudaSuccess) return cuda_fail(e, "mlp hidden launch");
     e = head_forward(ctx, u, B, F, head.W2, head.b2, head.centers, K, nullptr, 0.f, sp,
                      reinterpret_cast<float*>(ws + off_z), nullptr, nullptr, pred, probs, true, st);
@@ -483,7 +531,7 @@ estp_status launch_mlp_head_loss(estp_ctx* ctx, const float* pooled, int B, int6
     float* dz = reinterpret_cast<float*>(ws + off_dz);
     float2* part = reinterpret_cast<float2*>(ws + off_part);
     const bool lower = g.W1 || g.b1 || g.pooled;  // gradients below the hidden layer
-    cudaError_t e = wide_gemm<true, true>(ctx, side_rows(pooled, B, D), side_rows(head.W1, F, D), D, head.b1, u, false, st);
+    cudaError_t e = hidden_layer(ctx, pooled, B, D, head, u, st);
     if (e != cudaSuccess) return cuda_fail(e, "mlp hidden launch");
     e = head_forward(ctx, u, B, F, head.W2, head.b2, head.centers, K, targets, lambda3, sp,
                      reinterpret_cast<float*>(ws + off_z), dz, part, nullptr, nullptr, true, st);

@@ -114,11 +114,6 @@ namespace {
 // normalisers 485 -> 158 us, column sums 857 -> 162.
 constexpr int kFThreads = 256;
 constexpr int kFCols = 128;          // rows of a streamed tile
-// Items per SM below which the split gets finer.  4 prompts of 300 to 1500 tokens, 16 heads, d 128
-// (2.5 items of 128 rows per SM): row normalisers 158 us with 128 rows, 171 with 64.  Column sums at
-// 4 and at 8 items per SM: 164 and 162 us there, 432 and 369 on 32 prompts of 100 to 1000.
-constexpr int kFLseItemsPerSm = 2, kFImpItemsPerSm = 8;
-
 template <int TM, int TN>
 using ScoreTile = SgemmTile<TM, TN, 16, true, true, false>;
 constexpr int kFSmem = ScoreTile<8, 8>::kSmemFloats;
@@ -373,32 +368,9 @@ __global__ void imp_finalize_kernel(const float* acc, const int32_t* cu, int B, 
     out[j] = n > 0 ? acc[j] * inv_lh / (float)n : 0.f;
 }
 
-// Rows of an fp32 item's fixed side, query tiles per column-sum item, and whether each head
-// gets column-sum items of its own (else a KV group's heads share them).
-struct F32Split {
-    int rows, qc;
-    bool per_head;
-};
-
-int f32_rows(int B, int64_t sumT, int n_heads, int num_sms) {
-    return (int64_t)B * n_heads * mean_tiles(B, sumT, 128) >= (int64_t)kFLseItemsPerSm * num_sms ? 128 : 64;
-}
-
 // Whether a plan sorts its prompts: where some items wait for others to end.  (Below that the
 // sorting and the look-up cost ~2 us and give nothing.)
 int f32_sorted(int B, int64_t items, int64_t blocks) { return B > 1 && B <= kMaxSorted && items > blocks; }
-
-F32Split f32_split(int B, int64_t sumT, const ImpHeads& hs, int num_sms) {
-    F32Split s{128, 8, false};
-    auto enough = [&] {
-        const int64_t lists = (int64_t)B * (s.per_head ? hs.n_heads : hs.n_groups);
-        return lists * items_f(mean_tiles(B, sumT, s.rows), s.qc) >= (int64_t)kFImpItemsPerSm * num_sms;
-    };
-    if (!enough()) s.per_head = true;
-    while (!enough() && s.qc > 1) s.qc /= 2;
-    if (!enough()) s.rows = 64;
-    return s;
-}
 
 // A group of its own for every head.
 ImpHeads heads_apart(const ImpHeads& hs, int rep) {
@@ -472,13 +444,12 @@ estp_status launch_importance(estp_ctx* ctx, const void* Q, const void* K, estp_
                               int max_seqlen, bool accumulate, uint32_t flags, float* acc,
                               cudaStream_t st) {
     const bool tc = tc_supported(dtype, d);
-    const F32Split split = f32_split(B, sumT, heads, ctx->num_sms);
+    const F32Split split = f32_split(B, sumT, max_seqlen, heads.n_heads, heads.n_groups, ctx->num_sms);
     const bool apart = !tc && split.per_head;
     const ImpHeads hs = apart ? heads_apart(heads, Hq / Hkv) : heads;
     const int tile = tc ? tc_tile() : split.rows;
     const int qc = tc ? tc_qc(B, sumT, hs.n_groups, ctx->num_sms) : split.qc;
-    const int nt_max = (max_seqlen + tile - 1) / tile;
-    const int c_max = nt_max > 0 ? chunks_of(nt_max, 0, qc) : 0;
+    const int c_max = chunk_slots(max_seqlen, tile, qc);
     // workspace: [own lse][plan of the lse][plan][partials]
     const size_t lse_bytes = lse ? 0 : align_up(sizeof(float) * (size_t)Hq * (size_t)sumT, 256);
     const size_t off_lse_plan = lse_bytes;

@@ -44,6 +44,52 @@ inline int imp_pairs(int B, int64_t sumT, int n_groups, int pair, int num_sms) {
     return lists * items_f(nt, 1) <= num_sms ? 1 : 2;
 }
 
+// Chunk slots of the partial column sums, for prompts of up to `longest` tokens.
+inline int chunk_slots(int64_t longest, int tile, int qc) { return (int)div_up(div_up(longest, tile), qc); }
+
+// fp32 inputs.  Items per SM below which the split gets finer.  4 prompts of 300 to 1500 tokens, 16
+// heads, d 128 (2.5 items of 128 rows per SM): row normalisers 158 us with 128 rows, 171 with 64.
+// Column sums at 4 and at 8 items per SM: 164 and 162 us there, 432 and 369 on 32 prompts of 100 to 1000.
+constexpr int kFLseItemsPerSm = 2, kFImpItemsPerSm = 8;
+
+inline int f32_rows(int B, int64_t sumT, int n_heads, int num_sms) {
+    return (int64_t)B * n_heads * mean_tiles(B, sumT, 128) >= (int64_t)kFLseItemsPerSm * num_sms ? 128 : 64;
+}
+
+// Rows of an item's fixed side, query tiles per column-sum item, and whether each head gets
+// column-sum items of its own (else a KV group's heads share them).
+struct F32Split {
+    int rows, qc;
+    bool per_head;
+};
+
+// Finer splits keep more partial sums (a slot per chunk of query tiles and list of items): they are
+// taken while those fit kFPartBytes, or what chunks of 512 queries and one list per KV group would
+// take.  Without a limit a batch of many short prompts beside a long one, or a loose bound on their
+// length, takes up to 8 x heads per group as much as that.
+constexpr int64_t kFPartBytes = 64ll << 20;
+inline int64_t f32_part_bytes(const F32Split& s, int64_t sumT, int64_t longest, int n_heads, int n_groups) {
+    return 4 * (int64_t)chunk_slots(longest, s.rows, s.qc) * (s.per_head ? n_heads : n_groups) * sumT;
+}
+inline F32Split f32_split(int B, int64_t sumT, int64_t longest, int n_heads, int n_groups, int num_sms) {
+    F32Split s{128, 8, false};
+    const int64_t coarse = f32_part_bytes({64, 8, false}, sumT, longest, n_heads, n_groups);
+    const int64_t limit = coarse > kFPartBytes ? coarse : kFPartBytes;
+    // takes the split t if more items are wanted and it fits
+    const auto finer = [&](F32Split t) {
+        const int64_t lists = (int64_t)B * (s.per_head ? n_heads : n_groups);
+        if (lists * items_f(mean_tiles(B, sumT, s.rows), s.qc) >= (int64_t)kFImpItemsPerSm * num_sms) return false;
+        if (f32_part_bytes(t, sumT, longest, n_heads, n_groups) > limit) return false;
+        s = t;
+        return true;
+    };
+    finer({s.rows, s.qc, true});
+    while (s.qc > 1 && finer({s.rows, s.qc / 2, s.per_head})) {
+    }
+    finer({64, s.qc, s.per_head});
+    return s;
+}
+
 // ---------------------------------------------------------------- entropy from hidden states
 // n_rb row blocks x S vocabulary splits are dealt round-robin to one CTA an SM.  A split is cut in
 // cuts of `gran` units (32 entries) and worked off in tiles of kLmTileUnits; a tile that is not full

@@ -19,6 +19,13 @@ extern "C" void lm(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t sms, int
     *S = r.S;
     *gran = r.gran;
 }
+extern "C" int64_t part_bytes(int B, int64_t sumT, int64_t longest, int n_heads, int n_groups, int sms) {
+    return f32_part_bytes(f32_split(B, sumT, longest, n_heads, n_groups, sms), sumT, longest, n_heads, n_groups);
+}
+extern "C" int split(int B, int64_t sumT, int64_t longest, int n_heads, int n_groups, int sms) {
+    const F32Split s = f32_split(B, sumT, longest, n_heads, n_groups, sms);
+    return s.rows * 100 + s.qc * 10 + (s.per_head ? 1 : 0);
+}
 extern "C" int64_t ranges(int64_t sumT, int64_t row_bytes, int B, int64_t full, int n_slices, int sms) {
     return pool_ranges(sumT, row_bytes, B, full, n_slices, sms);
 }
@@ -109,6 +116,48 @@ def test_column_sum_items_of_one_pair_fit_the_sms(rules, n_groups):
             else:  # two pairs wherever one pair would not fit and longer items would leave SMs idle
                 assert B * n_groups * _items(nt, 1) > SMS, (B, T)
                 assert qc == 2 or items >= 16 * SMS, (B, T)
+
+
+# ------------------------------------------------------------------- column sums (fp32)
+@pytest.mark.parametrize("n_heads,n_groups", [(8, 8), (16, 4), (28, 4), (64, 8), (256, 1), (1, 1)])
+def test_f32_partials_stay_bounded(rules, n_heads, n_groups):
+    """No more than 64 MiB, or what chunks of 512 queries for each KV group take, however skewed the
+    lengths and however loose the bound on them (at most the whole batch)."""
+    i = ctypes.c_int64
+    rules.part_bytes.restype = i
+    for B in (1, 2, 8, 64, 256, 1000, 5000):
+        for T in (1, 16, 100, 300, 1000, 4000):
+            sumT = B * T
+            for longest in {T, min(sumT, 8 * T), min(sumT, 131072)}:
+                got = rules.part_bytes(B, i(sumT), i(longest), n_heads, n_groups, SMS)
+                coarse = 4 * _up(_up(longest, 64), 8) * n_groups * sumT
+                assert got <= max(coarse, 64 << 20), (B, T, longest, got, coarse)
+
+
+def _f32_unlimited(B, sumT, n_heads, n_groups):
+    rows, qc, per_head = 128, 8, False
+
+    def enough():
+        nt = _up(_up(sumT, B), rows)
+        return B * (n_heads if per_head else n_groups) * _items(nt, qc) >= 8 * SMS
+
+    per_head = per_head or not enough()
+    while not enough() and qc > 1:
+        qc //= 2
+    if not enough():
+        rows = 64
+    return rows, qc, per_head
+
+
+@pytest.mark.parametrize("n_heads,n_groups", [(8, 8), (16, 4), (28, 4), (1, 1)])
+def test_f32_split_follows_the_items_within_the_bound(rules, n_heads, n_groups):
+    i = ctypes.c_int64
+    for B in (1, 2, 4, 32, 160):
+        for T in (1, 16, 128, 300, 900, 1500, 4000):
+            rows, qc, per_head = _f32_unlimited(B, B * T, n_heads, n_groups)
+            if 4 * _up(_up(T, rows), qc) * (n_heads if per_head else n_groups) * B * T <= 64 << 20:
+                got = rules.split(B, i(B * T), i(T), n_heads, n_groups, SMS)
+                assert got == rows * 100 + qc * 10 + per_head, (B, T)
 
 
 # ---------------------------------------------------------------------------- pooling

@@ -28,6 +28,7 @@
 
 #include "estp_internal.cuh"
 #include "sgemm.cuh"
+#include "split_rules.cuh"
 
 namespace estp {
 namespace {
@@ -266,10 +267,8 @@ __global__ void __launch_bounds__(256, 2) wide_gemm_kernel(GemmSide A, GemmSide 
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)blockIdx.z, ranks = (int)gridDim.z;  // the cluster spans z
     const int64_t n0 = (int64_t)blockIdx.x * T::BN, m0 = (int64_t)blockIdx.y * T::BM;
-    const int64_t per = ((n_k + ranks - 1) / ranks + 63) / 64 * 64;
-    const int64_t k0 = rank * per, k1 = k0 + per < n_k ? k0 + per : n_k;
     T t;
-    t.run(sm, A, m0, Bm, n0, k0, k1);
+    t.run(sm, A, m0, Bm, n0, rank_begin(n_k, BK, rank, ranks), rank_begin(n_k, BK, rank + 1, ranks));
 #pragma unroll
     for (int i = 0; i < TM; ++i)
         *reinterpret_cast<float4*>(sm + t.row(i) * SC + t.col(0)) =
@@ -441,16 +440,14 @@ cudaError_t layer_grads(const float* x, int B, int64_t D, const float* W, int K,
 }
 
 // out [M, N] of wide_gemm_kernel.  The tile height follows M (a batch of prompts), so that a
-// small batch does not multiply padding; the cluster is the widest that keeps every rank two
-// slices of work and the grid within two blocks an SM.
+// small batch does not multiply padding; the cluster's width: wide_ranks.
 template <bool kAlongB, bool kRelu>
 cudaError_t wide_gemm(estp_ctx* ctx, const GemmSide& A, const GemmSide& Bm, int64_t n_k, const float* bias,
                       float* out, bool dependent, cudaStream_t st) {
     const int64_t M = A.rows, N = Bm.rows;
     const int tm = M > 64 ? 8 : M > 32 ? 4 : M > 16 ? 2 : 1;
     const dim3 tiles((unsigned)ceil_div(N, 64), (unsigned)ceil_div(M, 16 * tm));
-    int S = 8;
-    while (S > 1 && ((int64_t)tiles.x * tiles.y * S > 2 * (int64_t)ctx->num_sms || n_k / S < 128)) S /= 2;
+    const int S = wide_ranks((int64_t)tiles.x * tiles.y, n_k, ctx->num_sms);
     const dim3 grid(tiles.x, tiles.y, (unsigned)S);
     auto go = [&](auto kern) { return launch(kern, grid, 256, st, dependent, S, A, Bm, n_k, bias, out); };
     return tm == 8 ? go(wide_gemm_kernel<8, 16, kAlongB, kRelu>)

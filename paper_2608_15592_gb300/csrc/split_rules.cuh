@@ -163,4 +163,21 @@ inline int64_t pool_ranges(int64_t sumT, int64_t row_bytes, int B, int64_t full,
     return G > 1 ? G : 1;  // every range holds >= 1 token
 }
 
+// --------------------------------------------------------------------- wide products of the MLP
+// First value of rank `rank`'s share of a contraction of n_k values in slices of bk: whole slices,
+// as even as they go, so the longest share is one slice longer than the shortest at most.
+ESTP_RULE int64_t rank_begin(int64_t n_k, int bk, int rank, int ranks) {
+    const int64_t k = div_up(n_k, bk) * rank / ranks * bk;
+    return k < n_k ? k : n_k;
+}
+
+// Ranks (a power of two up to 8) along the contraction for `tiles` output tiles: as many as keep the
+// grid within two blocks an SM and every rank kRankValues values of the contraction.
+constexpr int kRankValues = 128;
+inline int wide_ranks(int64_t tiles, int64_t n_k, int num_sms) {
+    int S = 8;
+    while (S > 1 && (tiles * S > 2 * (int64_t)num_sms || n_k / S < kRankValues)) S /= 2;
+    return S;
+}
+
 }  // namespace estp

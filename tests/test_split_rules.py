@@ -26,6 +26,8 @@ extern "C" int split(int B, int64_t sumT, int64_t longest, int n_heads, int n_gr
     const F32Split s = f32_split(B, sumT, longest, n_heads, n_groups, sms);
     return s.rows * 100 + s.qc * 10 + (s.per_head ? 1 : 0);
 }
+extern "C" int64_t begin(int64_t n_k, int bk, int rank, int ranks) { return rank_begin(n_k, bk, rank, ranks); }
+extern "C" int ranks(int64_t tiles, int64_t n_k, int sms) { return wide_ranks(tiles, n_k, sms); }
 extern "C" int64_t ranges(int64_t sumT, int64_t row_bytes, int B, int64_t full, int n_slices, int sms) {
     return pool_ranges(sumT, row_bytes, B, full, n_slices, sms);
 }
@@ -180,3 +182,18 @@ def test_pool_ranges_balance_the_sms(rules, row_bytes, ctas_per_sm, n_slices):
                 # enough ranges in flight for the bytes, few enough slots to merge
                 want = (sumT * row_bytes * B / 4000) ** 0.5
                 assert 0.45 * want <= G <= want, (B, T, G)
+
+
+# ----------------------------------------------------------------- wide products (MLP head)
+@pytest.mark.parametrize("bk", [16, 32, 64])
+def test_no_rank_of_a_wide_product_idles(rules, bk):
+    i = ctypes.c_int64
+    rules.begin.restype = i
+    for n_k in [1, 15, 64, 127, 128, 255, 256, 1000, 1023, 1024, 1088, 1600, 2050, 4096, 5000, 8192, 12345]:
+        for tiles in (1, 16, 38, 39, 76, 77, 152, 153, 1000):
+            S = rules.ranks(i(tiles), i(n_k), SMS)
+            assert S in (1, 2, 4, 8) and (S == 1 or (tiles * S <= 2 * SMS and n_k / S >= 128))
+            cut = [rules.begin(i(n_k), bk, r, S) for r in range(S + 1)]
+            assert cut[0] == 0 and cut[-1] == n_k and all(c % bk == 0 for c in cut[:-1])
+            slices = [_up(b - a, bk) for a, b in zip(cut, cut[1:])]
+            assert max(slices) - min(slices) <= 1 and min(slices) >= 1, (n_k, S, slices)

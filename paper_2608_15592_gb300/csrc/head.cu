@@ -439,6 +439,9 @@ cudaError_t layer_grads(const float* x, int B, int64_t D, const float* W, int K,
     return launch(layer_grad_kernel, dim3((unsigned)(a.n_w + a.n_x + 1)), 256, st, true, 1, a);
 }
 
+// Rows of tiles of `side` rows that one launch covers: the y extent of a grid stops at 65535.
+int64_t rows_a_launch(int side) { return (int64_t)65535 * side; }
+
 // out [M, N] of wide_gemm_kernel.  The tile height follows M (a batch of prompts), so that a
 // small batch does not multiply padding; the cluster's width: wide_ranks.
 template <bool kAlongB, bool kRelu>
@@ -446,14 +449,21 @@ cudaError_t wide_gemm(estp_ctx* ctx, const GemmSide& A, const GemmSide& Bm, int6
                       float* out, bool dependent, cudaStream_t st) {
     const int64_t M = A.rows, N = Bm.rows;
     const int tm = M > 64 ? 8 : M > 32 ? 4 : M > 16 ? 2 : 1;
-    const dim3 tiles((unsigned)ceil_div(N, 64), (unsigned)ceil_div(M, 16 * tm));
-    const int S = wide_ranks((int64_t)tiles.x * tiles.y, n_k, ctx->num_sms);
-    const dim3 grid(tiles.x, tiles.y, (unsigned)S);
-    auto go = [&](auto kern) { return launch(kern, grid, 256, st, dependent, S, A, Bm, n_k, bias, out); };
-    return tm == 8 ? go(wide_gemm_kernel<8, 16, kAlongB, kRelu>)
-         : tm == 4 ? go(wide_gemm_kernel<4, 32, kAlongB, kRelu>)
-         : tm == 2 ? go(wide_gemm_kernel<2, 32, kAlongB, kRelu>)
-                   : go(wide_gemm_kernel<1, 64, kAlongB, kRelu>);
+    const int S = wide_ranks((int64_t)ceil_div(N, 64) * ceil_div(M, 16 * tm), n_k, ctx->num_sms);
+    cudaError_t e = cudaSuccess;
+    for (int64_t m = 0; m < M && e == cudaSuccess; m += rows_a_launch(16 * tm)) {
+        const int64_t rows = M - m < rows_a_launch(16 * tm) ? M - m : rows_a_launch(16 * tm);
+        const GemmSide a{A.p + m * A.ld, A.ld, rows, A.vec};
+        const dim3 grid((unsigned)ceil_div(N, 64), (unsigned)ceil_div(rows, 16 * tm), (unsigned)S);
+        auto go = [&](auto kern) {
+            return launch(kern, grid, 256, st, dependent || m > 0, S, a, Bm, n_k, bias, out + m * N);
+        };
+        e = tm == 8 ? go(wide_gemm_kernel<8, 16, kAlongB, kRelu>)
+          : tm == 4 ? go(wide_gemm_kernel<4, 32, kAlongB, kRelu>)
+          : tm == 2 ? go(wide_gemm_kernel<2, 32, kAlongB, kRelu>)
+                    : go(wide_gemm_kernel<1, 64, kAlongB, kRelu>);
+    }
+    return e;
 }
 
 // The hidden layer u = max(W1 h + b1, 0), the first launch of its call.
@@ -537,9 +547,14 @@ estp_status launch_mlp_head_loss(estp_ctx* ctx, const float* pooled, int B, int6
     e = layer_grads(u, B, F, head.W2, K, dz, part, lambda3, loss, g.W2, g.b2, lower ? gu : nullptr, u, st);
     if (e != cudaSuccess) return cuda_fail(e, "mlp second-layer gradient launch");
     if (g.W1 || g.b1) {  // first layer: dL/dW1, dL/db1
-        const GemmSide h = side_cols(pooled, D);
-        e = launch(outer_kernel, dim3((unsigned)(g.W1 ? ceil_div(D, OuterTile::BN) : 1), (unsigned)ceil_div(F, OuterTile::BM)),
-                   256, st, true, 1, side_cols(gu, F), h, (int64_t)B, h.vec && (!g.W1 || aligned16(g.W1)) ? 1 : 0, g.W1, g.b1);
+        const GemmSide h = side_cols(pooled, D), gs = side_cols(gu, F);
+        const int vec = h.vec && (!g.W1 || aligned16(g.W1)) ? 1 : 0;
+        for (int64_t f = 0; f < F && e == cudaSuccess; f += rows_a_launch(OuterTile::BM)) {
+            const int64_t rows = F - f < rows_a_launch(OuterTile::BM) ? F - f : rows_a_launch(OuterTile::BM);
+            e = launch(outer_kernel, dim3((unsigned)(g.W1 ? ceil_div(D, OuterTile::BN) : 1), (unsigned)ceil_div(rows, OuterTile::BM)),
+                       256, st, true, 1, GemmSide{gs.p + f, gs.ld, rows, gs.vec}, h, (int64_t)B, vec,
+                       g.W1 ? g.W1 + f * D : nullptr, g.b1 ? g.b1 + f : nullptr);
+        }
         if (e != cudaSuccess) return cuda_fail(e, "mlp first-layer gradient launch");
     }
     if (g.pooled) {  // dL/dpooled = W1^T g

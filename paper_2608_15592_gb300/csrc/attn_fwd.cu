@@ -603,7 +603,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // C_j (+)= sum over heads h and query tiles qt >= kt(j) of the partial slots of key j.  A block
 // takes 32 keys; its warp w sums heads w, w + 16, .. (each over qt in eights), and the 16 warp
 // sums are added as a tree: a fixed order, whatever the launch.  16 prompts of 256 to 2048 tokens,
-// 28 heads: 220.8 us for forward and reduce, 223.6 with 8 warps, 224.7 with 32.
+// 28 heads: 220.8 us for forward and reduce, 223.6 with 8 warps, 224.7 with 32.  64 prompts of 16 to
+// 100 tokens, 28 and 32 heads: 47.3 and 52.0 us, 49.6 and 55.4 with 8 warps.
 constexpr int kRedHeadLanes = 16;
 __global__ void __launch_bounds__(32 * kRedHeadLanes)
     imp_fwd_reduce_kernel(const float* __restrict__ part, const int32_t* cu, const int32_t* base2,

@@ -285,7 +285,8 @@ __global__ void __launch_bounds__(kMergeThreads) entropy_merge_kernel(EntArgs a,
 }
 
 // Threads of a row in the merge, for its number of pieces: a row of up to two is merged by one
-// thread (each extra lane costs more than it reads), one of more than a warp by a block.
+// thread (each extra lane costs more than it reads), one of up to 64 by at most a warp, one of
+// more by a block.
 int merge_lanes(int64_t n_warps, int64_t n_rows) {
     if (n_warps <= 2 * n_rows) return 1;
     if (n_warps > 64 * n_rows) return kMergeThreads;

@@ -1,8 +1,8 @@
 // Attention importance (Eq. 2-0, Sec. 3.1): row log-normalisers, causal column sums
 // of the softmax attention, the deterministic partial reduce and the final scaling.
 //
-// This file holds the device plan, the CUDA-core kernels (fp32 inputs, and any
-// shape the tensor-core path does not take) and the launchers that pick a path.
+// This file holds the device plan, the CUDA-core kernels for fp32 inputs (bf16 inputs go to the
+// tensor cores at both head sizes) and the launchers that pick a path.
 //
 // Column sums are formed in the transposed orientation: a CTA owns a tile of KEYS
 // and streams the query tiles that may attend to it, so the sum over queries of

@@ -16,7 +16,7 @@
 // Integer counts: the result is exact.
 //
 // What bounds it is latency: each pass is one look at the prompt's keys (those of its first 2048
-// tokens in registers, the rest from L1), three barriers and a scan.  While the two intervals of a
+// tokens in registers, the rest from L1), four barriers and a scan.  While the two intervals of a
 // value agree, which they do in the first pass, one histogram serves both: half of the shared
 // atomics.  256 prompts of 128 to 4096 tokens: 144 us for 32 passes of 8-bit digits, one selection
 // at a time, each scanned by one thread; 23.0 for the passes above with every key re-read and four

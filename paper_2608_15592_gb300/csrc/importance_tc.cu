@@ -369,8 +369,10 @@ __global__ void __launch_bounds__(threads_of(MODE), 1)
                     const uint32_t u = step / C::kStages;
                     const int y = si.y, row0 = si.row0, head = si.head;
                     // the next item is claimed before this one's last copies, which hide the
-                    // round trip of the atomic
-                    if (s == t.n_steps - 1) item = (int)gridDim.x + atomicAdd(&info->next, 1);
+                    // round trip of the atomic (where there are no more items than CTAs it would
+                    // delay the only copies: 0.4 us of the 7 a one-step call takes)
+                    if (s == t.n_steps - 1)
+                        item = total > (int)gridDim.x ? (int)gridDim.x + atomicAdd(&info->next, 1) : total;
                     if (MODE == kModeImp) {  // the tile's lse values, from a 16-byte boundary
                         const int ls = (int)(step % kLseSlots);
                         const uint32_t lu = step / kLseSlots;

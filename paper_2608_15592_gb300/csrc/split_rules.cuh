@@ -149,11 +149,14 @@ inline LmSplit lm_split(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t num
 // 20.7 with 152, 22.9 with 304; 8 x 700 x 4096 26.9 with 303, 22.6 with 152, 24.7 with 304.  (Smaller
 // CTAs are limited by their own loads: 16 x 256..2048 x 512 bf16 20.7 us with 281, 25.5 with 152.)  A
 // wave that would be five sixths full is filled: 64 x 512 x 512 fp32 18.9 us with 1036, 18.6 with 1216.
+// Up to kPoolTokens tokens each have a range of their own, as a second row in one costs more than its
+// slot: 16 x 4096 bf16, cold, 18.4 us with 15 ranges or 6, 16.9 with 16.
 constexpr double kPoolRangeBytes = 4000.0;
+constexpr int64_t kPoolTokens = 16;
 inline int64_t pool_ranges(int64_t sumT, int64_t row_bytes, int B, int64_t full, int n_slices, int num_sms) {
     int64_t G = full;
     const double few = sqrt((double)sumT * (double)row_bytes * B / kPoolRangeBytes);
-    if ((double)G > few) {
+    if (sumT > kPoolTokens && (double)G > few) {
         G = (int64_t)few;
         const int64_t two = 2 * (int64_t)num_sms;
         if (full * n_slices <= two && G * n_slices > num_sms && G * n_slices < two) G = num_sms / n_slices;

@@ -174,6 +174,8 @@ def test_pool_ranges_balance_the_sms(rules, row_bytes, ctas_per_sm, n_slices):
             sumT = B * T
             G = rules.ranges(i(sumT), i(row_bytes), B, i(full), n_slices, SMS)
             assert 1 <= G <= min(full, sumT), (B, T)
+            if sumT <= 16:
+                assert G == min(full, sumT), (B, T, G)
             ctas = G * n_slices
             if sumT >= full and G < full:
                 # no SM with two large CTAs among SMs with one, and no wave that is nearly full

@@ -113,7 +113,7 @@ struct LmSplit {
 // the rule's S is within 1.8 % of the best one.  A rule that took the first S whose last round is
 // 97 % full, of at most four times the fewest, left SMs idle or took rounds that cost more than
 // they filled: 14848 rows, D 896, V 128256 2370 us for S = 1 against 2154 for 5; 20000 rows, D 4096,
-// V 8000 996 against 902; 5888 rows, D 4096, V 128256 4004 for S = 13 against 3851 for 6.
+// V 8000 996 against 850; 5888 rows, D 4096, V 128256 4004 for S = 13 against 3851 for 6.
 constexpr int kLmPassShare = 64;
 
 // s_min: at least as many splits as keep the row blocks in flight in L2.

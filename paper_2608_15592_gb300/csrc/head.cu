@@ -263,12 +263,15 @@ __global__ void __launch_bounds__(256, 2) wide_gemm_kernel(GemmSide A, GemmSide 
     using T = WideTile<TM, BK, kAlongB>;
     constexpr int SC = T::BN + 4;
     __shared__ __align__(16) float sm[T::kSmemFloats > T::BM * SC ? T::kSmemFloats : T::BM * SC];
-    chain_launches();
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)blockIdx.z, ranks = (int)gridDim.z;  // the cluster spans z
     const int64_t n0 = (int64_t)blockIdx.x * T::BN, m0 = (int64_t)blockIdx.y * T::BM;
+    // the share's divisions before the wait for the launch before this one: 64 prompts, D and F 1024,
+    // training step 48.2 us with them after it, 46.7
+    const int64_t k0 = rank_begin(n_k, BK, rank, ranks), k1 = rank_begin(n_k, BK, rank + 1, ranks);
+    chain_launches();
     T t;
-    t.run(sm, A, m0, Bm, n0, rank_begin(n_k, BK, rank, ranks), rank_begin(n_k, BK, rank + 1, ranks));
+    t.run(sm, A, m0, Bm, n0, k0, k1);
 #pragma unroll
     for (int i = 0; i < TM; ++i)
         *reinterpret_cast<float4*>(sm + t.row(i) * SC + t.col(0)) =

@@ -26,6 +26,8 @@
 //   for kernels that read an operand from L2 for every few FMAs; the call 1016 -> 198 us.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "estp_internal.cuh"
 #include "sgemm.cuh"
 #include "split_rules.cuh"
@@ -328,7 +330,7 @@ __global__ void __launch_bounds__(256, 2) outer_kernel(GemmSide g, GemmSide h, i
 }
 
 // u[b, f] = max(sum_x W1[f, x] h[b, x] + b1[f], 0) for a batch of at most NB prompts: one warp a
-// hidden unit, lanes along D four columns at a time, then a fixed butterfly.  With so few prompts
+// hidden unit, lanes along D, then a fixed butterfly.  With so few prompts
 // reading W1 is the bound, and a tile of wide_gemm_kernel has only a slice of it in flight (one
 // prompt, 4096 x 1024: 31 us cold, which is 0.5 TB/s).  Prediction through the MLP, F 1024, with that
 // kernel and with this one: 1 prompt, D 4096, 32 bins 35.7 and 18.5 us; 4 prompts, D 8192, 128 bins
@@ -345,18 +347,29 @@ __global__ void __launch_bounds__(128) hidden_rows_kernel(GemmSide h, GemmSide w
     float2 acc[NB][2];
 #pragma unroll
     for (int j = 0; j < NB; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
-    for (int64_t x = 4 * lane; x < D; x += 128) {
-        // every load of the pass first (prompts past the batch read as zero), then the FMAs
-        const float4 wv = LogitTile::fetch<true>(w, f, x, D);
-        float4 hv[NB];
+    // a lane takes four of every 128 columns: neighbouring ones, in one load, where the rows allow it
+    // (D then is a multiple of 4), else each 32 apart, so that a load covers 128 bytes of the row
+    const auto add = [&](auto vec) {
+        const auto four = [&](const float* row, int64_t x) {
+            if constexpr (decltype(vec)::value) return *reinterpret_cast<const float4*>(row + x);
+            return make_float4(row[x], x + 32 < D ? row[x + 32] : 0.f, x + 64 < D ? row[x + 64] : 0.f,
+                               x + 96 < D ? row[x + 96] : 0.f);
+        };
+        for (int64_t x = decltype(vec)::value ? 4 * lane : lane; x < D; x += 128) {
+            // every load of the pass first (prompts past the batch count as zero), then the FMAs
+            const float4 wv = four(w.p + f * w.ld, x);
+            float4 hv[NB];
 #pragma unroll
-        for (int j = 0; j < NB; ++j) hv[j] = LogitTile::fetch<true>(h, j, x, D);
+            for (int j = 0; j < NB; ++j) hv[j] = j < h.rows ? four(h.p + j * h.ld, x) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
-            acc[j][0] = __ffma2_rn(make_float2(wv.x, wv.y), make_float2(hv[j].x, hv[j].y), acc[j][0]);
-            acc[j][1] = __ffma2_rn(make_float2(wv.z, wv.w), make_float2(hv[j].z, hv[j].w), acc[j][1]);
+            for (int j = 0; j < NB; ++j) {
+                acc[j][0] = __ffma2_rn(make_float2(wv.x, wv.y), make_float2(hv[j].x, hv[j].y), acc[j][0]);
+                acc[j][1] = __ffma2_rn(make_float2(wv.z, wv.w), make_float2(hv[j].z, hv[j].w), acc[j][1]);
+            }
         }
-    }
+    };
+    if (h.vec && w.vec) add(std::true_type{});
+    else add(std::false_type{});
     const float b = bias ? bias[f] : 0.f;
 #pragma unroll
     for (int j = 0; j < NB; ++j) {

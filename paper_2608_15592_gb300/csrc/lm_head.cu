@@ -63,8 +63,7 @@ struct LmArgs {
     long long wait_cycles;  // limit of the abortable waits (kWaitCycles unless a test lowers it)
 };
 
-// Vocabulary units [u0, u1) of split sp: lm_split says when splits end inside a tile.  Such a last
-// tile loads and multiplies only the units it has.
+// Vocabulary units [u0, u1) of split sp: lm_split says when splits end inside a tile.
 __device__ __forceinline__ void split_range(const LmArgs& a, int sp, int& u0, int& u1) {
     const int64_t n = (a.n_unit + a.gran - 1) / a.gran;
     u0 = (int)(sp * n / a.S) * a.gran;
@@ -188,9 +187,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                             break;
                         }
                         uint8_t* st = sm + stage * kStageBytes;
-                        mbar_expect_tx(&full[stage], a.a_bytes + n_u * (kBBytes / kTileUnits));
+                        // a tile of a split of whole tiles is one box, past the vocabulary zero-filled; another
+                        // one's last tile is a box for each of its units
+                        const int boxed = n_u == kTileUnits || a.gran == kTileUnits ? kTileUnits : n_u;
+                        mbar_expect_tx(&full[stage], a.a_bytes + boxed * (kBBytes / kTileUnits));
                         tma_load_2d(st, &tm_a, kc * kKc, rb * kM, &full[stage]);
-                        if (n_u == kTileUnits) {
+                        if (boxed == kTileUnits) {
                             tma_load_2d(st + kABytes, &tm_b, kc * kKc, ut * kUnit, &full[stage]);
                         } else {
                             for (int j = 0; j < n_u; ++j)

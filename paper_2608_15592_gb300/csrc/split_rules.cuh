@@ -92,12 +92,7 @@ inline F32Split f32_split(int B, int64_t sumT, int64_t longest, int n_heads, int
 
 // ---------------------------------------------------------------- entropy from hidden states
 // n_rb row blocks x S vocabulary splits are dealt round-robin to one CTA an SM.  A split is cut in
-// cuts of `gran` units (32 entries) and worked off in tiles of kLmTileUnits; a tile that is not full
-// takes as long as a full one or longer (its A box is loaded all the same, and its W box unit by
-// unit), so splits are whole tiles.  Only where W is the bound (a single row block: every CTA streams
-// its own share) or where whole tiles do not give every SM an item are they cut in units, which are
-// equal within one.  Whole tiles against units, the same S: 20000 rows, D 4096, V 8000 850 and 920
-// us; 3000 rows there 140 and 142; 256 rows, V 32000 72.2 and 80.3; one row, V 128256 180.7 and 176.6.
+// cuts of `gran` units (32 entries), 8 (a whole tile) or 1, and worked off in tiles of kLmTileUnits.
 constexpr int kLmTileUnits = 8;
 
 struct LmSplit {
@@ -105,34 +100,48 @@ struct LmSplit {
     int gran;
 };
 
-// S minimises, for the SM with the most items, its cuts plus what each item costs beside them, over
-// up to 16 items an SM (or four times the fewest).  An item costs its share of one more pass of W
-// through L2: with S forced it came to a 40th to a 100th of the vocabulary.  Of the splits with the
-// same number of items an SM the largest is the best, so one per number is looked at.  Measured
-// sustained over 37 sizes (129 to 21663 rows, D 896 to 4096, V 5000 to 152064) with 8 to 10 S each:
-// the rule's S is within 1.8 % of the best one.  A rule that took the first S whose last round is
-// 97 % full, of at most four times the fewest, left SMs idle or took rounds that cost more than
-// they filled: 14848 rows, D 896, V 128256 2370 us for S = 1 against 2154 for 5; 20000 rows, D 4096,
-// V 8000 996 against 850; 5888 rows, D 4096, V 128256 4004 for S = 13 against 3851 for 6.
-constexpr int kLmPassShare = 64;
+// Time of an item of u units, in tenths of a full tile's unit.  A tile of r < 8 units loads a box of
+// W for each of them beside its box of hidden states, which one thread issues: about 2 + 1.6 r units'
+// time (from items of 2 to 10 tiles with S forced; 5 units cost more than a whole tile).
+inline int64_t lm_item_cost(int64_t u) {
+    const int64_t r = u % kLmTileUnits;
+    return 10 * (u - r) + (r ? 20 + 16 * r : 0);
+}
+
+// Of the cuts in units and in whole tiles, and of the numbers of splits that give the busiest SM w
+// items (the largest S of each, up to 16 items or four times the fewest), the one that is least for
+// that SM: its items plus, for each, 1 / kLmPassShare of the vocabulary.  That is what an item costs
+// beside its tiles, its share of one more pass of W through L2 (a 40th to a 100th of the vocabulary
+// with S forced; from a 40th to an 80th the rule's choices are equally good).  A single row block is cut in units: streaming W is the bound there and the
+// shares have to be equal (one row, V 128256: 176.6 us, 180.7 in whole tiles).
+// Measured sustained over 37 sizes (129 to 21663 rows, D 896 to 4096, V 5000 to 152064) with 8 to 10
+// S each: whole tiles with the rule's S are within 1.8 % of the best S.  A rule that took the first S
+// in units whose last round is 97 % full, of at most four times the fewest, left SMs idle or took
+// rounds that cost more than they filled: 14848 rows, D 896, V 128256 2374 us for S = 1 against 2123
+// for 5; 20000 rows, D 4096, V 8000 1005 against 843; 5888 rows, D 4096, V 128256 3937 for S = 13
+// against 3801 for 6.
+constexpr int kLmPassShare = 80;
 
 // s_min: at least as many splits as keep the row blocks in flight in L2.
 inline LmSplit lm_split(int64_t n_rb, int64_t n_unit, int64_t s_min, int64_t num_sms) {
     const int64_t n_tile = div_up(n_unit, kLmTileUnits);
-    const bool whole = n_rb > 1 && n_rb * n_tile >= num_sms;
-    const int64_t n = whole ? n_tile : n_unit;
-    LmSplit best{n < s_min ? n : s_min, whole ? kLmTileUnits : 1};
-    const int64_t w0 = div_up(n_rb * best.S, num_sms);  // items of the busiest SM
-    const int64_t w1 = 4 * w0 > 16 ? 4 * w0 : 16;
+    LmSplit best{1, 1};
     int64_t best_cost = INT64_MAX;
-    for (int64_t w = w0; w <= w1; ++w) {
-        const int64_t S = w * num_sms / n_rb < n ? w * num_sms / n_rb : n;
-        const int64_t cost = div_up(n_rb * S, num_sms) * (kLmPassShare * div_up(n, S) + n);
-        if (cost < best_cost) {
-            best_cost = cost;
-            best.S = S;
+    for (int gran = n_rb > 1 ? kLmTileUnits : 1; gran >= 1; gran -= kLmTileUnits - 1) {
+        const int64_t n = gran > 1 ? n_tile : n_unit;
+        const int64_t w0 = div_up(n_rb * (n < s_min ? n : s_min), num_sms);  // items of the busiest SM
+        const int64_t w1 = 4 * w0 > 16 ? 4 * w0 : 16;
+        for (int64_t w = w0; w <= w1; ++w) {
+            const int64_t S = w * num_sms / n_rb < n ? w * num_sms / n_rb : n;
+            int64_t cost = div_up(n_rb * S, num_sms) *
+                           (lm_item_cost(div_up(n, S) * gran) + 10 * n_unit / kLmPassShare);
+            if (gran == 1) cost += cost / 50;  // units only for a gain beyond the model's error
+            if (cost < best_cost) {
+                best_cost = cost;
+                best = LmSplit{S, gran};
+            }
+            if (S == n) break;
         }
-        if (S == n) break;
     }
     return best;
 }
